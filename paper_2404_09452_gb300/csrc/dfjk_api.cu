@@ -17,6 +17,7 @@
 #include "common.cuh"
 #include "grad.cuh"
 #include "integrals.cuh"
+#include "ksplit.cuh"
 #include "linalg.cuh"
 #include "ozaki.cuh"
 #include "pool.cuh"
@@ -272,6 +273,17 @@ struct XWork {
 };
 constexpr size_t C_SLICE_CAP = (size_t)1 << 30;
 
+// Buffers of the K GEMM over sliced operands, sized once for the longest reduction
+// range (alloc_kwork): graphs and queued builds keep their addresses.
+struct KWork {
+  DBuf<double> part;  // partial sums of the splits
+  DBuf<int> seq;      // split counters of the ordered kernel
+  void release() {
+    part.release();
+    seq.release();
+  }
+};
+
 // Launch-shape choices that do not change what is computed, only how fast:
 // rows per block of the slicing kernels, the K GEMM's split-K range and the
 // mixed build's work-buffer cap (which sets the aux-row chunk).  0 = the
@@ -360,7 +372,6 @@ struct dfjk_ctx {
   DBuf<double> V, L, Linv, Dinv;
   DBuf<int> status;
   DBuf<int> tctr;  // tile counter of the tensor-core GEMM launches (stream-ordered)
-  DBuf<int> kseq;  // split counters of the ordered split-K GEMM
   // whitened tensor B, P contiguous: DFJK_FP64 keeps both triangles,
   // B[(mu nao + nu) ldb + P]; DFJK_MIXED keeps one row per kept column m (the
   // whitening's output order), B[m ldb + P], found through rowmap, and slices
@@ -388,6 +399,7 @@ struct dfjk_ctx {
   DBuf<int> rowmap;  // DFJK_MIXED: row of B for AO pair (mu, nu), -1 if screened
   int ksplit = 1;
   SlicedOp Xsl;  // slices of X, the K GEMM's operand
+  KWork kw;
   DBuf<double> uks_D, uks_J;  // spin-unrestricted build: D_a + D_b and J[D_b]
   cudaStream_t side = nullptr;  // setup: Cholesky + inverse beside the integrals
   cudaStream_t side2 = nullptr;  // the Cholesky's bulk trailing updates (look-ahead)
@@ -1008,6 +1020,7 @@ void release_device(dfjk_ctx *h) {
   h->rho_work.release();
   h->X.release();
   h->Kpart.release();
+  h->kw.release();
   h->en_work.release();
   h->e.release();
   oz_free(h->Xsl);
@@ -1111,6 +1124,31 @@ void x_gemm_sliced(dfjk_ctx *h, const PairLists &pl, const int *expo, XWork &w, 
   }
 }
 
+size_t k_range_bytes(int range_mb) {
+  static const size_t env = [] {
+    const char *e = std::getenv("DFJK_K_RANGE_MB");
+    const long v = e ? std::atol(e) : 0;
+    return (size_t)(v > 0 ? v : 64) << 20;
+  }();
+  return range_mb > 0 ? (size_t)range_mb << 20 : env;
+}
+
+// The K GEMM of operands with nao rows in format fmt.
+KShape k_shape(int nao, int fmt, int range_mb) {
+  KShape s;
+  s.nao = nao;
+  s.tiles = k_tiles(nao, OZ_BM, OZ_BN);
+  s.block_bytes = (size_t)ceil_div(nao, OZ_BM) * OZ_BM * oz_slices(fmt) * 2 * oz_kblock(fmt);
+  s.range_bytes = k_range_bytes(range_mb);
+  s.ordered = !oz_simple_mode();
+  return s;
+}
+
+void alloc_kwork(KWork &w, const KShape &s, int fmt, long long kt) {
+  w.part.alloc(k_part_doubles(s, ceil_div(kt, oz_kblock(fmt))));
+  w.seq.alloc(oz_tile_seq_count(s.nao, s.nao));
+}
+
 // Build buffers, sized on the first build at a given nocc and reused after.
 void ensure_workspace(dfjk_ctx *h, int nocc, int nset) {
   const size_t nao2 = (size_t)h->nao * h->nao;
@@ -1124,6 +1162,7 @@ void ensure_workspace(dfjk_ctx *h, int nocc, int nset) {
       h->rho_work.alloc((size_t)RHO_PARTS * h->naux_pad);
       oz_alloc(h->Xsl, 1, h->bfmt, h->nao, pc * nocc, OZ_BM);
       alloc_xwork(h, h->pl, h->xw, pc, nocc);
+      alloc_kwork(h->kw, k_shape(h->nao, h->bfmt, h->tune.k_range_mb), h->bfmt, (long long)pc * nocc);
     } else {
       h->rho_work.alloc(std::max((size_t)128 * ceil_div(h->naux_pad, 256) * 256, (size_t)h->nao * h->naux_pad));
       h->X.alloc((size_t)h->nao * h->naux_pad * nocc);
@@ -1170,45 +1209,25 @@ void add_inplace(double *y, const double *x, long long n, cudaStream_t st) {
 // splits per tile, and the chain of adds (about 3 us each) was longer than the
 // products (an FP64 density build at 8 atoms 3.95 -> 0.77 ms, a build at 5 atoms 331
 // -> 226 us).  The one-tile-per-CTA kernel always writes partials.
-constexpr size_t K_PART_BYTES = (size_t)64 << 20;
-void k_gemm_sliced(dfjk_ctx *h, const SlicedOp &xs, const SlicedOp &ys, int nao, long long kt, double *Kout, bool add,
-                   cudaStream_t st) {
-  const int mt = ceil_div(nao, OZ_BM), nt = ceil_div(nao, OZ_BN);
-  int tiles = 0;
-  for (int i = 0; i < mt; ++i)
-    for (int j = 0; j < nt; ++j)
-      if (j * OZ_BN <= i * OZ_BM + OZ_BM - 1) ++tiles;
-  static const size_t range_env = [] {
-    const char *e = std::getenv("DFJK_K_RANGE_MB");
-    const long v = e ? std::atol(e) : 0;
-    return (size_t)(v > 0 ? v : 64) << 20;
-  }();
-  const size_t range_bytes = h->tune.k_range_mb > 0 ? (size_t)h->tune.k_range_mb << 20 : range_env;
-  const int nkb = xs.nkb;
-  const size_t chunk_kb_bytes = (size_t)xs.rows_pad * xs.S * 2 * oz_kblock(xs.fmt);
-  int per = (int)std::max<size_t>(1, range_bytes / chunk_kb_bytes);
-  const bool ordered = !oz_simple_mode();
-  const int max_split = ordered ? nkb : (int)std::max<size_t>(1, ((size_t)4 << 30) / ((size_t)nao * nao * 8));
-  int nsplit = std::min(ceil_div(nkb, per), max_split);
-  nsplit = std::max(nsplit, std::min(nkb, (2 * 152 + tiles - 1) / tiles));
-  per = ceil_div(nkb, nsplit);
-  nsplit = ceil_div(nkb, per);
-  const size_t part = (size_t)nsplit * nao * nao;
+// `w`: from alloc_kwork for at least this range.
+void k_gemm_sliced(dfjk_ctx *h, KWork &w, const SlicedOp &xs, const SlicedOp &ys, int nao, long long kt, double *Kout,
+                   bool add, cudaStream_t st) {
+  const KShape s = k_shape(nao, xs.fmt, h->tune.k_range_mb);
+  const KSplit p = k_split(s, xs.nkb);
+  if (p.partials ? w.part.n < (size_t)p.n * nao * nao : w.seq.n < oz_tile_seq_count(nao, nao))
+    throw Error{DFJK_ERR_STATE, "K work buffers"};
   OzGemmArgs k;
-  k.M = nao; k.N = nao; k.K = (int)kt; k.nz = nsplit; k.kb_per_split = per; k.lower_only = 1;
+  k.M = nao; k.N = nao; k.K = (int)kt; k.nz = p.n; k.kb_per_split = p.per; k.lower_only = 1;
   k.status = h->status.p; k.timeout = h->opt.timeout_iters;
   k.tile_ctr = h->tctr.p;
   k.phase = 10;
-  if (ordered && part * sizeof(double) > K_PART_BYTES) {
-    const size_t nseq = oz_tile_seq_count(nao, nao);
-    if (h->kseq.n < nseq) h->kseq.alloc(nseq);
-    k.mode = 2; k.out = Kout; k.ldo = nao; k.tile_seq = h->kseq.p; k.accumulate = add ? 1 : 0;
+  if (!p.partials) {
+    k.mode = 2; k.out = Kout; k.ldo = nao; k.tile_seq = w.seq.p; k.accumulate = add ? 1 : 0;
     oz_gemm(xs, ys, k, st);
   } else {
-    if (h->Kpart.n < part) h->Kpart.alloc(part);
-    k.mode = 0; k.out = h->Kpart.p; k.ldo = nao; k.out_bs = (long long)nao * nao;
+    k.mode = 0; k.out = w.part.p; k.ldo = nao; k.out_bs = (long long)nao * nao;
     oz_gemm(xs, ys, k, st);
-    reduce_sym_f64(h->Kpart.p, nsplit, nao, Kout, st, add ? 1 : 0);
+    reduce_sym_f64(w.part.p, p.n, nao, Kout, st, add ? 1 : 0);
   }
 }
 
@@ -1321,7 +1340,7 @@ void build_one(dfjk_ctx *h, int nocc, const double *C, double *J, double *Kout, 
       PhaseScope ph(5, st);
       SlicedOp xs = oz_view(h->Xsl, nao, (int)kt);  // rows mu, K (p, i)
       oz_slice_f64(Xc, 0, kt, 1, xs, st, h->tune.slice_rows);
-      k_gemm_sliced(h, xs, xs, nao, kt, Kout, c > 0, st);
+      k_gemm_sliced(h, h->kw, xs, xs, nao, kt, Kout, c > 0, st);
     }
     mirror_lower_f64(Kout, nao, st);
     if (sj != st) DFJK_CUDA_CHECK(cudaStreamWaitEvent(st, h->ev_join, 0));  // D and J ready
@@ -1341,6 +1360,7 @@ struct DensityWork {
   DBuf<int> expo_own;
   const int *expo = nullptr;
   XWork xw;
+  KWork kw;
   SlicedOp xs, bs;
   int ns = 0, pc = 0;  // sigma and rows P per chunk
   ~DensityWork() {
@@ -1385,6 +1405,7 @@ void density_work(dfjk_ctx *h, DensityWork &w, cudaStream_t st) {
   oz_alloc(w.xs, 1, OZ_F64, nao, w.ns * np, OZ_BM);
   oz_alloc(w.bs, 1, OZ_F64, nao, w.ns * np, OZ_BM);
   alloc_xwork(h, w.pl, w.xw, w.pc, w.ns);
+  alloc_kwork(w.kw, k_shape(nao, OZ_F64, h->tune.k_range_mb), OZ_F64, (long long)w.ns * np);
 }
 
 // K = sum_P B_P D B_P on the tensor cores, for ranges of sigma: W[mu][sigma][P] =
@@ -1418,7 +1439,7 @@ void density_k_sliced(dfjk_ctx *h, DensityWork &w, const double *D, double *Kout
     oz_slice_f64(w.W.p, 0, kt, 1, xs, st, h->tune.slice_rows);
     if (!keep_b)
       oz_slice_f64(w.Bf + (long long)s0 * h->ldb, 0, (long long)nao * h->ldb, 1, bs, st, h->tune.slice_rows);
-    k_gemm_sliced(h, xs, bs, nao, kt, Kout, s0 > 0, st);
+    k_gemm_sliced(h, w.kw, xs, bs, nao, kt, Kout, s0 > 0, st);
   }
   mirror_lower_f64(Kout, nao, st);
 }
@@ -1595,6 +1616,7 @@ int dfjk_estimate_bytes(int32_t nao, int32_t naux, int32_t nocc, int32_t precisi
     ws += oz_pairs_bytes(fmt, (long long)steps, (int)pc);                 // B slices
     const size_t cs = c_step_bytes(fmt, nocc);                            // C slices
     ws += std::min(std::max(C_SLICE_CAP, rup(n, OZ_BK) / OZ_BK * cs), steps * cs);
+    ws += k_part_doubles(k_shape(nao, fmt, 0), (int)nkb) * 8 + oz_tile_seq_count(nao, nao) * 4;  // K partials
   } else {
     const size_t t = (n + 63) / 64, ksplit = std::max<size_t>(1, std::min<size_t>(64, (4 * 152 + t * (t + 1) / 2 - 1) / (t * (t + 1) / 2)));
     ws += n * np * no * 8 + n * n * ksplit * 8 + n * np * 8;  // X, K partials, rho partials
