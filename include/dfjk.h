@@ -233,8 +233,7 @@ int dfjk_build(dfjk_handle h, int32_t nset, int32_t nocc, const double *C_occ,
  * Uses a work buffer of nao^2 naux_pad doubles for the duration of the call,
  * and for a DFJK_MIXED handle (B of the kept pairs only) a second one holding
  * B in both triangles of every pair; synchronises the stream before
- * returning.  Errors:
- * DFJK_ERR_ARG, _OOM, _CUDA.                            */
+ * returning.  Errors: DFJK_ERR_ARG, _OOM, _TIMEOUT, _CUDA.                   */
 int dfjk_build_density(dfjk_handle h, int32_t nset, const double *D, double *J, double *K,
                        double *E_J, double *E_K, void *stream);
 
@@ -272,7 +271,7 @@ int dfjk_coulomb_gradient(dfjk_handle h, const double *D, double *grad, void *st
  *   C_occ : device nao x nocc FP64 row-major, 1 <= nocc <= nao.
  *   c_j, c_k : finite weights of E_J and E_K (c_k = 0 skips the K part).
  *   grad : device natom x 3 FP64, overwritten.
- * Synchronises the stream.  Errors: DFJK_ERR_ARG, _OOM, _CUDA.               */
+ * Synchronises the stream.  Errors: DFJK_ERR_ARG, _OOM, _TIMEOUT, _CUDA.     */
 int dfjk_jk_gradient(dfjk_handle h, int32_t nocc, const double *C_occ, double c_j, double c_k, double *grad,
                      void *stream);
 

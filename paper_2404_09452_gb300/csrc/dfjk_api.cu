@@ -1177,6 +1177,17 @@ void ensure_workspace(dfjk_ctx *h, int nocc, int nset) {
   if (!h->e.p || h->e.n < (size_t)(2 * nset)) h->e.alloc(2 * nset);
 }
 
+// After the stream of a call has been synchronised: an expired bounded wait left part of
+// its results unwritten.  The status bit is cleared, so that the next call starts afresh.
+void throw_on_timeout(dfjk_ctx *h, const char *what) {
+  int status = 0;
+  DFJK_CUDA_CHECK(cudaMemcpy(&status, h->status.p, sizeof(int), cudaMemcpyDeviceToHost));
+  if (status & STATUS_TIMEOUT) {
+    DFJK_CUDA_CHECK(cudaMemset(h->status.p, 0, sizeof(int)));
+    throw Error{DFJK_ERR_TIMEOUT, std::string("a bounded device wait expired during the ") + what};
+  }
+}
+
 __global__ void split_energies_kernel(const double *e, int nset, double *EJ, double *EK) {
   const int s = threadIdx.x + blockIdx.x * blockDim.x;
   if (s < nset) {
@@ -1696,12 +1707,7 @@ int dfjk_build(dfjk_handle h, int32_t nset, int32_t nocc, const double *C, doubl
         EJ[s] = e[2 * s];
         EK[s] = e[2 * s + 1];
       }
-      int status = 0;  // the stream is synchronised here: surface device status
-      DFJK_CUDA_CHECK(cudaMemcpy(&status, h->status.p, sizeof(int), cudaMemcpyDeviceToHost));
-      if (status & STATUS_TIMEOUT) {
-        DFJK_CUDA_CHECK(cudaMemset(h->status.p, 0, sizeof(int)));
-        throw Error{DFJK_ERR_TIMEOUT, "a bounded device wait expired during the build"};
-      }
+      throw_on_timeout(h, "build");
     } else {
       split_energies_kernel<<<ceil_div(nset, 64), 64, 0, st>>>(h->e.p, nset, EJ, EK);
       DFJK_LAUNCHED();
@@ -1755,12 +1761,7 @@ int dfjk_build_uks(dfjk_handle h, int32_t nocc_a, const double *C_a, int32_t noc
       E[0] = host[4];
       E[1] = host[1];
       E[2] = host[3];
-      int status = 0;
-      DFJK_CUDA_CHECK(cudaMemcpy(&status, h->status.p, sizeof(int), cudaMemcpyDeviceToHost));
-      if (status & STATUS_TIMEOUT) {
-        DFJK_CUDA_CHECK(cudaMemset(h->status.p, 0, sizeof(int)));
-        throw Error{DFJK_ERR_TIMEOUT, "a bounded device wait expired during the build"};
-      }
+      throw_on_timeout(h, "build");
     }
     return DFJK_OK;
   } catch (const Error &e) {
@@ -1817,6 +1818,7 @@ int dfjk_build_density(dfjk_handle h, int32_t nset, const double *D, double *J, 
         EK[s] = e[2 * s + 1];
       }
     }
+    throw_on_timeout(h, "density build");
     return DFJK_OK;
   } catch (const Error &e) {
     return fail(e);
@@ -2044,12 +2046,7 @@ static void jk_gradient(dfjk_ctx *h, const double *Din, int nocc, const double *
     }
   }
   DFJK_CUDA_CHECK(cudaStreamSynchronize(st));  // local buffers are released on return
-  int status = 0;
-  DFJK_CUDA_CHECK(cudaMemcpy(&status, h->status.p, sizeof(int), cudaMemcpyDeviceToHost));
-  if (status & STATUS_TIMEOUT) {
-    DFJK_CUDA_CHECK(cudaMemset(h->status.p, 0, sizeof(int)));
-    throw Error{DFJK_ERR_TIMEOUT, "a bounded device wait expired during the gradient"};
-  }
+  throw_on_timeout(h, "gradient");
 }
 
 int dfjk_coulomb_gradient(dfjk_handle h, const double *D, double *grad, void *stream) {
