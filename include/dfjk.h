@@ -86,9 +86,9 @@ typedef enum {
                     kept in both triangles, nao^2 naux_pad doubles            */
   DFJK_MIXED = 1 /* 3-centre integrals and their derivatives in
                     double-single arithmetic (two FP32 numbers, about 48 bits;
-                    FP64 for exponents outside 1e-4 .. 1e4 or atoms more than
-                    256 bohr from the centroid; FP32 for the pairs below
-                    fp32_pair_thresh), the metric, Cholesky and inverse, rho, J
+                    FP64 for exponents outside 1e-4 .. 1e4, atoms more than
+                    256 bohr from the centroid or fp32_pair_thresh = 0; FP32
+                    for the pairs below fp32_pair_thresh), the metric, Cholesky and inverse, rho, J
                     and the energies in FP64.  B is kept in FP64 for the
                     Schwarz-kept AO pairs only, one row of naux_pad doubles
                     per kept column (a quarter of the mu >= nu pairs at 60
@@ -119,9 +119,11 @@ typedef struct {
                               "Limitations and Future Development"): kept
                               pairs whose bound sqrt(max(ab|ab)) *
                               max_P sqrt((P|P)) is below this value are
-                              evaluated in FP32.  0 = every pair in FP64;
-                              negative = the precision's default (0 for
-                              DFJK_FP64, 1e-5 for DFJK_MIXED)                 */
+                              evaluated in FP32.  0 = every pair in FP64, its
+                              derivatives too (a DFJK_MIXED handle then uses
+                              no double-single arithmetic); negative = the
+                              precision's default (0 for DFJK_FP64, 1e-5 for
+                              DFJK_MIXED)                                     */
   int32_t b_on_host;       /* 1: keep B in pinned host memory mapped into the
                               device address space (the kernels read and
                               write it in place over the host link; for

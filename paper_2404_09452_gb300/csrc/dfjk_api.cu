@@ -346,7 +346,8 @@ struct dfjk_ctx {
   DBuf<double> o_center, o_exps, o_coefs, a_center, a_exps, a_cdiv, a_g1;
   DBuf<float2> a_df;   // aux centres (from c0), exponents, cdiv, g1 as double-single pairs
   double c0[3] = {0.0, 0.0, 0.0};  // centroid
-  bool use_df = false;  // the FP64 pairs' integrals in double-single (df_range_ok)
+  bool df_range = false;  // a mixed handle whose exponents and coordinates suit FP32 pairs (df_range_ok)
+  bool use_df = false;  // its integrals in double-single, unless fp32_pair_thresh = 0 asks for FP64
   DBuf<int> o_prim_off, o_nprim, o_func_off, a_prim_off, a_nprim, a_func_off;
   DBuf<int> aux_cls[3];
   std::vector<int> aux_cls_n = std::vector<int>(3, 0);
@@ -804,7 +805,7 @@ void make_resident(dfjk_ctx *h, cudaStream_t st) {
     PairClassArgs a{n, h->pair_a.p + b0, h->pair_b.p + b0, h->pair_rec_off.p + b0, h->rec.p, h->q.p + b0,
                     h->pair_npp.p + b0};
     launch_pair_kernel(cls[c][0], cls[c][1], a, orb_args(h), tab, st);
-    launch_schwarz(cls[c][0], cls[c][1], a, tab, tab32, h->use_df, st);
+    launch_schwarz(cls[c][0], cls[c][1], a, tab, tab32, h->df_range, st);
   }
   h->scal.alloc(1);
   max_sqrt_diag(h->V.p, h->naux, np, h->scal.p, st);
@@ -1572,7 +1573,8 @@ int dfjk_setup(const dfjk_basis *orb, const dfjk_basis *aux, int32_t natom, cons
       h->c0[d] = 0.0;
       for (int a = 0; a < natom; ++a) h->c0[d] += h->coords[3 * (size_t)a + d] / natom;
     }
-    h->use_df = h->opt.precision == DFJK_MIXED && df_range_ok(h);
+    h->df_range = h->opt.precision == DFJK_MIXED && df_range_ok(h);
+    h->use_df = h->df_range && h->opt.fp32_pair_thresh != 0.0;
     h->opt.tune_table = nullptr;  // the caller's string is not kept
     make_resident(h, S(stream));
     *out = h;
