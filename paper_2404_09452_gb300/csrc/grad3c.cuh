@@ -579,11 +579,8 @@ inline int grad_chunk(int npairs, int aux_blocks) {
 template <int LAB, int LC, typename Real>
 void launch_grad3c_j(GradArgs a, const AuxArgs &x, const typename EriIn<Real>::Tab *tab, cudaStream_t st) {
   using Sh = GradShape<LAB, LC, false, Real, GRAD_HDR + 6 * ntuv(LAB + 1)>;
-  static bool attr = false;
-  if (!attr) {
-    DFJK_CUDA_CHECK(cudaFuncSetAttribute(grad3c_j_kernel<LAB, LC, Real>, cudaFuncAttributeMaxDynamicSharedMemorySize, Sh::SMEM));
-    attr = true;
-  }
+  static OncePerDevice once;
+  allow_smem(once, grad3c_j_kernel<LAB, LC, Real>, Sh::SMEM);
   const int ny = ceil_div(a.naux_shells, Sh::NS);
   a.pair_chunk = grad_chunk(a.npairs, ny);
   grad3c_j_kernel<LAB, LC, Real><<<dim3(ceil_div(a.npairs, a.pair_chunk), ny), Sh::THREADS, Sh::SMEM, st>>>(a, x, tab);
@@ -592,11 +589,8 @@ void launch_grad3c_j(GradArgs a, const AuxArgs &x, const typename EriIn<Real>::T
 template <int LA, int LB, int LC, typename Real>
 void launch_grad3c_x(GradArgs a, const AuxArgs &x, const typename EriIn<Real>::Tab *tab, cudaStream_t st) {
   using Sh = GradShape<LA + LB, LC, true, Real, GRAD_HDR + 4 * nterms(LA, LB)>;
-  static bool attr = false;
-  if (!attr) {
-    DFJK_CUDA_CHECK(cudaFuncSetAttribute(grad3c_x_kernel<LA, LB, LC, Real>, cudaFuncAttributeMaxDynamicSharedMemorySize, Sh::SMEM));
-    attr = true;
-  }
+  static OncePerDevice once;
+  allow_smem(once, grad3c_x_kernel<LA, LB, LC, Real>, Sh::SMEM);
   const int ny = ceil_div(a.naux_shells, Sh::NS);
   a.pair_chunk = grad_chunk(a.npairs, ny);
   grad3c_x_kernel<LA, LB, LC, Real><<<dim3(ceil_div(a.npairs, a.pair_chunk), ny), Sh::THREADS, Sh::SMEM, st>>>(a, x, tab);
