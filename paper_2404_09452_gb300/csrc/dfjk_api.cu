@@ -389,7 +389,7 @@ struct dfjk_ctx {
   std::vector<int> pl_h;  // list, gstep, zstep and zgroup, in this order
   std::vector<int> gstep_h, gfirst_h;  // host copies: K steps before a group, its first AO
   XWork xw;
-  DBuf<double> b_stage;  // B in host memory: a chunk's columns of B on the device
+  DBuf<double> b_stage;  // B in host memory: the columns of B of a build's chunk on the device
   int chunk_rows = 0;   // rows P per build chunk (sliced products)
   DBuf<int> Bexpo;      // slice exponents of B's slices, [mu][expo_rows][pl.nkb]
   int expo_rows = 0;    // rows P of Bexpo (naux_pad rounded up to 128)
@@ -689,16 +689,22 @@ void upload_pair_lists(dfjk_ctx *h, cudaStream_t st) {
   oz_krow(pl, h->lean ? h->rowmap.p : nullptr, h->nao, h->pl_krow.p, st);
 }
 
+// Doubles of `pc` columns of B, for every row.
+size_t stage_size(const dfjk_ctx *h, int pc) {
+  return std::max<size_t>(1, h->lean ? (size_t)h->ncol : (size_t)h->nao * h->nao) * pc;
+}
 // Columns [p0, p0 + pc) of a host-resident B, for every row, on the device (rows
-// of pc doubles): the kernels that slice B read each pair twice.
-void stage_columns(dfjk_ctx *h, int p0, int pc, cudaStream_t st) {
+// of pc doubles): the kernels that slice B read each pair twice.  `buf` has been
+// sized by its owner: a buffer that moved here would leave a captured or queued
+// build behind with the old one.
+const double *stage_columns(dfjk_ctx *h, const DBuf<double> &buf, int p0, int pc, cudaStream_t st) {
   const size_t rows = h->lean ? (size_t)h->ncol : (size_t)h->nao * h->nao;
-  const size_t need = std::max<size_t>(rows, 1) * pc;
-  if (h->b_stage.n < need) h->b_stage.alloc(need);
+  if (buf.n < stage_size(h, pc)) throw Error{DFJK_ERR_STATE, "staging buffer of B"};
   if (rows)
-    DFJK_CUDA_CHECK(cudaMemcpy2DAsync(h->b_stage.p, (size_t)pc * sizeof(double), h->B.p + p0,
+    DFJK_CUDA_CHECK(cudaMemcpy2DAsync(buf.p, (size_t)pc * sizeof(double), h->B.p + p0,
                                       (size_t)h->ldb * sizeof(double), (size_t)pc * sizeof(double), rows,
                                       cudaMemcpyDefault, st));
+  return buf.p;
 }
 
 // rho and J over the kept columns of B, stored as rows m (lean) or mu nao + nu.
@@ -975,14 +981,16 @@ void make_resident(dfjk_ctx *h, cudaStream_t st) {
     PhaseScope ph(3, st);
     const int nkb = h->pl.nkb;
     h->expo_rows = (np + OZ_BM - 1) / OZ_BM * OZ_BM;
+    DBuf<double> stage;
     h->Bexpo.alloc((size_t)h->nao * h->expo_rows * nkb);
     if (!h->B.host) {
       oz_expo_pairs(h->B.p, h->ldb, np, h->pl, h->nao, h->expo_rows, 0, h->expo_rows, h->Bexpo.p, st);
     } else {  // in chunks of columns, each copied to the device once
+      stage.alloc(stage_size(h, std::min(512, np)));
       for (int p0 = 0; p0 < h->expo_rows; p0 += 512) {
         const int pc = std::min(512, h->expo_rows - p0), live = std::max(0, std::min(pc, np - p0));
-        if (live > 0) stage_columns(h, p0, live, st);
-        oz_expo_pairs(h->b_stage.p, live, live, h->pl, h->nao, pc, p0, h->expo_rows, h->Bexpo.p, st);
+        if (live > 0) stage_columns(h, stage, p0, live, st);
+        oz_expo_pairs(stage.p, live, live, h->pl, h->nao, pc, p0, h->expo_rows, h->Bexpo.p, st);
       }
     }
     DFJK_CUDA_CHECK(cudaStreamSynchronize(st));
@@ -1163,6 +1171,7 @@ void ensure_workspace(dfjk_ctx *h, int nocc, int nset) {
       h->rho_work.alloc((size_t)RHO_PARTS * h->naux_pad);
       oz_alloc(h->Xsl, 1, h->bfmt, h->nao, pc * nocc, OZ_BM);
       alloc_xwork(h, h->pl, h->xw, pc, nocc);
+      if (h->B.host) h->b_stage.alloc(stage_size(h, pc));
       alloc_kwork(h->kw, k_shape(h->nao, h->bfmt, h->tune.k_range_mb), h->bfmt, (long long)pc * nocc);
     } else {
       h->rho_work.alloc(std::max((size_t)128 * ceil_div(h->naux_pad, 256) * 256, (size_t)h->nao * h->naux_pad));
@@ -1331,8 +1340,7 @@ void build_one(dfjk_ctx *h, int nocc, const double *C, double *J, double *Kout, 
       const double *b = h->B.p + p0;
       long long ldb = h->ldb;
       if (h->B.host) {  // one copy of the chunk's columns; rho of the chunk from it
-        stage_columns(h, p0, pc, st);
-        b = h->b_stage.p;
+        b = stage_columns(h, h->b_stage, p0, pc, st);
         ldb = pc;
         rho_of(b, ldb, p0, pc, st);
       }
@@ -1365,7 +1373,7 @@ void build_one(dfjk_ctx *h, int nocc, const double *C, double *J, double *Kout, 
 struct DensityWork {
   bool sliced = false;
   const double *Bf = nullptr;  // B with both triangles of every pair
-  DBuf<double> Bfull, W, Kpart;
+  DBuf<double> Bfull, W, Kpart, stage;
   int ksplit = 1;
   // sliced: X for a range of sigma, the slices of X and B, the lists and exponents
   PairLists pl;
@@ -1417,6 +1425,7 @@ void density_work(dfjk_ctx *h, DensityWork &w, cudaStream_t st) {
   oz_alloc(w.xs, 1, OZ_F64, nao, w.ns * np, OZ_BM);
   oz_alloc(w.bs, 1, OZ_F64, nao, w.ns * np, OZ_BM);
   alloc_xwork(h, w.pl, w.xw, w.pc, w.ns);
+  if (h->B.host) w.stage.alloc(stage_size(h, w.pc));
   alloc_kwork(w.kw, k_shape(nao, OZ_F64, h->tune.k_range_mb), OZ_F64, (long long)w.ns * np);
 }
 
@@ -1436,10 +1445,7 @@ void density_k_sliced(dfjk_ctx *h, DensityWork &w, const double *D, double *Kout
       for (int p0 = 0; p0 < np; p0 += w.pc) {
         const int pc = std::min(w.pc, np - p0);
         const double *b = h->B.p + p0;
-        if (h->B.host && !keep_a) {
-          stage_columns(h, p0, pc, st);
-          b = h->b_stage.p;
-        }
+        if (h->B.host && !keep_a) b = stage_columns(h, w.stage, p0, pc, st);
         x_gemm_sliced(h, w.pl, w.expo, w.xw,
                       XArgs{b, h->B.host ? pc : h->ldb, D + (long long)s0 * nao, 1, nao, ns, p0, pc, w.W.p + p0, np, kt, 3,
                             p0 == 0, keep_a || (w.pc >= np && s0 > 0)},
@@ -1889,7 +1895,7 @@ static void jk_gradient(dfjk_ctx *h, const double *Din, int nocc, const double *
     // molecules of DFJK_FP64
     const bool tc = h->sliced;
     const long long no2 = (long long)nocc * nocc;
-    DBuf<double> X, Xt, Z;
+    DBuf<double> X, Xt, Z, stage;
     XWork xw;
     X.alloc((size_t)nao * np * nocc);
     Xt.alloc((size_t)np * no2);
@@ -1903,13 +1909,11 @@ static void jk_gradient(dfjk_ctx *h, const double *Din, int nocc, const double *
       // as the build does
       const int pcm = build_chunk_rows(nao, np, nocc, h->bfmt, h->pl.steps, h->tune.build_ws_mb);
       alloc_xwork(h, h->pl, xw, pcm, nocc);
+      if (h->B.host) stage.alloc(stage_size(h, pcm));
       for (int p0 = 0; p0 < np; p0 += pcm) {
         const int pc = std::min(pcm, np - p0);
         const double *b = h->B.p + p0;
-        if (h->B.host) {
-          stage_columns(h, p0, pc, st);
-          b = h->b_stage.p;
-        }
+        if (h->B.host) b = stage_columns(h, stage, p0, pc, st);
         x_gemm_sliced(h, h->pl, h->Bexpo.p, xw,
                       XArgs{b, h->B.host ? pc : h->ldb, C, nocc, 1, nocc, p0, pc, X.p + (size_t)p0 * nocc, nocc,
                             (long long)np * nocc, 0, p0 == 0}, st);
