@@ -21,6 +21,7 @@
 #include "linalg.cuh"
 #include "ozaki.cuh"
 #include "pool.cuh"
+#include "stream_scope.cuh"
 
 namespace dfjk {
 
@@ -420,15 +421,6 @@ struct dfjk_ctx {
   }
 };
 
-// Waits for a stream on scope exit (error paths included), so that buffers the
-// stream still uses are not returned to the cache under it.
-struct StreamDrain {
-  cudaStream_t s;
-  ~StreamDrain() {
-    if (s) cudaStreamSynchronize(s);
-  }
-};
-
 namespace {
 
 cudaStream_t S(void *s) { return (cudaStream_t)s; }
@@ -764,8 +756,9 @@ void make_resident(dfjk_ctx *h, cudaStream_t st) {
     ~OzLocal() { oz_free(op); }
   } linv8_, t8_;
   SlicedOp &Linv8 = linv8_.op, &T8 = t8_.op;
-  DBuf<double> inv_work;
-  StreamDrain drain_side{s2}, drain_side2{h->side2}, drain_side3{h->side3};  // destroyed before the buffers above
+  DBuf<double> inv_work, stage;
+  DBuf<double> T;  // doubles, or double-single pairs (use_df)
+  StreamDrain drain{st}, drain_side{s2}, drain_side2{h->side2}, drain_side3{h->side3};  // destroyed before the buffers above
   {
     PhaseScope ph1(1, s2);
     h->L.alloc((size_t)np * np);
@@ -896,7 +889,6 @@ void make_resident(dfjk_ctx *h, cudaStream_t st) {
   const long long slab_budget = h->sliced ? (2LL << 30) : (4LL << 30);
   long long slab_cols = std::max<long long>(36, slab_budget / ((long long)np * 8));
   slab_cols = std::min<long long>(slab_cols, std::max<long long>(h->ncol, 1));
-  DBuf<double> T;  // doubles, or double-single pairs (use_df)
   T.alloc((size_t)slab_cols * np);
   DFJK_CUDA_CHECK(cudaMemsetAsync(T.p, 0, T.bytes(), st));
   if (h->use_df || h->npair_fp32 > 0) {
@@ -981,7 +973,6 @@ void make_resident(dfjk_ctx *h, cudaStream_t st) {
     PhaseScope ph(3, st);
     const int nkb = h->pl.nkb;
     h->expo_rows = (np + OZ_BM - 1) / OZ_BM * OZ_BM;
-    DBuf<double> stage;
     h->Bexpo.alloc((size_t)h->nao * h->expo_rows * nkb);
     if (!h->B.host) {
       oz_expo_pairs(h->B.p, h->ldb, np, h->pl, h->nao, h->expo_rows, 0, h->expo_rows, h->Bexpo.p, st);
@@ -1793,6 +1784,7 @@ int dfjk_build_density(dfjk_handle h, int32_t nset, const double *D, double *J, 
     en.alloc(2 * 256);
     if (!h->e.p || h->e.n < (size_t)(2 * nset)) h->e.alloc(2 * nset);
     DensityWork dw;
+    const StreamDrain drain{st};
     density_work(h, dw, st);
     for (int s = 0; s < nset; ++s) {
       const double *Ds = D + s * nao2;
@@ -1833,6 +1825,19 @@ int dfjk_build_density(dfjk_handle h, int32_t nset, const double *D, double *J, 
   }
 }
 
+// Buffers of a gradient call.
+struct GradWork {
+  DBuf<double> D, rho, work, d, X, Xt, Z, stage, W, gam;
+  DBuf<double> rec, gm;  // pair records and weights: doubles or double-single pairs
+  DBuf<long long> goff;
+  DBuf<int> orb_atom, aux_atom, aux_l;
+  XWork xw;
+  std::deque<SlicedOp> ops;  // slices of the tensor-core GEMMs
+  ~GradWork() {
+    for (SlicedOp &o : ops) oz_free(o);
+  }
+};
+
 // d(cj E_J + ck E_K)/dR at fixed D = C C^T (or the given D when ck = 0).
 // E = sum_PQ (V^-1)_PQ M_PQ / 2 for both energies, M_PQ = u_P u_Q (J) or
 // Tr(D T_P D T_Q) (K), so dE/dR = sum_P Tr(Gam_P dT_P/dR) - Tr(Wt dV/dR) / 2
@@ -1844,39 +1849,33 @@ static void jk_gradient(dfjk_ctx *h, const double *Din, int nocc, const double *
   if (!h->resident) make_resident(h, st);
   const int nao = h->nao, np = h->naux_pad;
   const double *tab = boys_table_device();
-  DBuf<double> Dl;
+  GradWork wk;
+  const StreamDrain drain{st};
   const double *D = Din;
   if (!D) {  // D = C C^T
-    Dl.alloc((size_t)nao * nao);
+    wk.D.alloc((size_t)nao * nao);
     GemmArgs dd;
     dd.M = nao; dd.N = nao; dd.K = nocc;
     dd.A = C; dd.sAm = nocc; dd.sAk = 1;
     dd.B = C; dd.sBn = nocc; dd.sBk = 1;
-    dd.C = Dl.p; dd.sCm = nao; dd.sCn = 1;
+    dd.C = wk.D.p; dd.sCm = nao; dd.sCn = 1;
     gemm_f64(dd, st);
-    D = Dl.p;
+    D = wk.D.p;
   }
   // rho = B vec D (= L^-1 u), then the fitted coefficients d = L^-T rho = V^-1 u
-  DBuf<double> rho, work, d;
+  DBuf<double> &rho = wk.rho, &work = wk.work, &d = wk.d;
   rho.alloc(np);
   work.alloc(std::max<size_t>((size_t)128 * ceil_div(np, 256) * 256, (size_t)16 * np));
   d.alloc(np);
   DFJK_CUDA_CHECK(cudaMemsetAsync(d.p, 0, d.bytes(), st));
   rho_kept(h, h->B.p, h->ldb, D, np, rho.p, work.p, st);
   fitted_coefficients(h->Linv.p, h->naux, np, rho.p, work.p, d.p, st);
-  DBuf<double> gam, W;
-  std::deque<SlicedOp> ops;  // slices of the tensor-core GEMMs, freed after the final sync
-  struct OpsFree {
-    std::deque<SlicedOp> &v;
-    ~OpsFree() {
-      for (SlicedOp &o : v) oz_free(o);
-    }
-  } ops_free{ops};
+  DBuf<double> &gam = wk.gam, &W = wk.W;
   // view x(z, r, k) = p[z sz + r sr + k sk] in sliced form
   auto slice = [&](const double *p, long long sz, long long sr, long long sk, int batch, int rows, int K,
                    int tile) -> SlicedOp & {
-    ops.emplace_back();
-    SlicedOp &o = ops.back();
+    wk.ops.emplace_back();
+    SlicedOp &o = wk.ops.back();
     oz_alloc(o, batch, h->bfmt, rows, K, tile);
     oz_slice_f64(p, sz, sr, sk, o, st);
     return o;
@@ -1895,8 +1894,8 @@ static void jk_gradient(dfjk_ctx *h, const double *Din, int nocc, const double *
     // molecules of DFJK_FP64
     const bool tc = h->sliced;
     const long long no2 = (long long)nocc * nocc;
-    DBuf<double> X, Xt, Z, stage;
-    XWork xw;
+    DBuf<double> &X = wk.X, &Xt = wk.Xt, &Z = wk.Z, &stage = wk.stage;
+    XWork &xw = wk.xw;
     X.alloc((size_t)nao * np * nocc);
     Xt.alloc((size_t)np * no2);
     Z.alloc((size_t)np * no2);
@@ -1975,9 +1974,11 @@ static void jk_gradient(dfjk_ctx *h, const double *Din, int nocc, const double *
       gm.C = gam.p; gm.sCm = nao; gm.sCn = 1; gm.sCb = (long long)nao * nao;
       gemm_f64(gm, st);
     }
-    DFJK_CUDA_CHECK(cudaStreamSynchronize(st));  // X, Xt, Z are released here
+    DFJK_CUDA_CHECK(cudaStreamSynchronize(st));
+    for (DBuf<double> *b : {&X, &Xt, &Z, &stage}) b->release();
+    xw.release();
   }
-  DBuf<int> oat, aat, al;
+  DBuf<int> &oat = wk.orb_atom, &aat = wk.aux_atom, &al = wk.aux_l;
   oat.upload(h->orb.atom, st);
   aat.upload(h->aux.atom, st);
   al.upload(h->aux.l, st);
@@ -2011,9 +2012,9 @@ static void jk_gradient(dfjk_ctx *h, const double *Din, int nocc, const double *
   for (int c = 0; c < 6; ++c)
     for (int i = h->kept_cls_begin[c]; i < h->kept_cls_begin[c + 1]; ++i)
       off[i + 1] = off[i] + (long long)h->npp_h[h->kept_h[i]] * grad_record_len(cls[c][0], cls[c][1], exch);
-  DBuf<long long> goff;
+  DBuf<long long> &goff = wk.goff;
   goff.upload(off, st);
-  DBuf<double> rec, gm;  // doubles or double-single pairs
+  DBuf<double> &rec = wk.rec, &gm = wk.gm;
   rec.alloc(std::max<size_t>(1, (size_t)off.back()));
   if (exch) gm.alloc((size_t)std::max<long long>(h->ncol, 1) * np);
   for (int c = 0; c < 6; ++c) {
@@ -2028,7 +2029,6 @@ static void jk_gradient(dfjk_ctx *h, const double *Din, int nocc, const double *
   // The classes run on the integral streams, the largest first: one after the other each
   // left the GPU to its own last wave: 45 atoms (Coulomb) 11.3 -> 9.7 ms,
   // 30 atoms (Coulomb and exchange) 19.2 -> 16.1.
-  StreamDrain drain{st};
   {
     const IntegralFork fork(st, h->ev_int);
     launch_grad2c(g, aux_args(h), al.p, h->aux.nshell, tab, fork.is[INT_STREAMS - 1]);
@@ -2051,7 +2051,7 @@ static void jk_gradient(dfjk_ctx *h, const double *Din, int nocc, const double *
       }
     }
   }
-  DFJK_CUDA_CHECK(cudaStreamSynchronize(st));  // local buffers are released on return
+  DFJK_CUDA_CHECK(cudaStreamSynchronize(st));
   throw_on_timeout(h, "gradient");
 }
 
