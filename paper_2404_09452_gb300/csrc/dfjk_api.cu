@@ -1252,10 +1252,8 @@ void build_one(dfjk_ctx *h, int nocc, const double *C, double *J, double *Kout, 
   // D, rho and J beside the tensor-core GEMMs, on the handle's side stream: they need
   // C and B only (rho = B vec D over the kept rows of B)
   const cudaStream_t sj = h->sliced && h->side ? h->side : st;
-  if (sj != st) {
-    DFJK_CUDA_CHECK(cudaEventRecord(h->ev_fork, st));
-    DFJK_CUDA_CHECK(cudaStreamWaitEvent(sj, h->ev_fork, 0));
-  }
+  SideScope side(st, sj, h->ev_fork, h->ev_join);
+  side.fork();
   GemmArgs d;  // D = C C^T
   d.M = nao; d.N = nao; d.K = nocc;
   d.A = C; d.sAm = nocc; d.sAk = 1;
@@ -1310,10 +1308,7 @@ void build_one(dfjk_ctx *h, int nocc, const double *C, double *J, double *Kout, 
       rho_of(h->B.p, h->ldb, 0, np, sj);
       j_of(sj);
     }
-    if (sj != st) {
-      DFJK_CUDA_CHECK(cudaEventRecord(h->ev_join, sj));
-      if (h->B.host) DFJK_CUDA_CHECK(cudaStreamWaitEvent(st, h->ev_join, 0));  // D ready
-    }
+    if (h->B.host) side.join();  // D ready
     const int pc_max = h->chunk_rows;
     const int nchunk = ceil_div(np, pc_max);
     // B does not change after setup: with one chunk its slices stay in the work
@@ -1341,12 +1336,8 @@ void build_one(dfjk_ctx *h, int nocc, const double *C, double *J, double *Kout, 
       }
       h->xw.b_ready = keep;
       if (h->B.host && c == nchunk - 1) {  // J beside the last K GEMM
-        if (sj != st) {
-          DFJK_CUDA_CHECK(cudaEventRecord(h->ev_fork, st));
-          DFJK_CUDA_CHECK(cudaStreamWaitEvent(sj, h->ev_fork, 0));
-        }
+        side.fork();
         j_of(sj);
-        if (sj != st) DFJK_CUDA_CHECK(cudaEventRecord(h->ev_join, sj));
       }
       PhaseScope ph(5, st);
       SlicedOp xs = oz_view(h->Xsl, nao, (int)kt);  // rows mu, K (p, i)
@@ -1354,7 +1345,7 @@ void build_one(dfjk_ctx *h, int nocc, const double *C, double *J, double *Kout, 
       k_gemm_sliced(h, h->kw, xs, xs, nao, kt, Kout, c > 0, st);
     }
     mirror_lower_f64(Kout, nao, st);
-    if (sj != st) DFJK_CUDA_CHECK(cudaStreamWaitEvent(st, h->ev_join, 0));  // D and J ready
+    side.join();  // D and J ready
   }
   PhaseScope ph(7, st);
   energies_f64(h->D.p, J, Kout, nao, e, h->en_work.p, st);

@@ -36,3 +36,32 @@ def test_drain_before_release(tmp_path, stream, throws):
     out = _run(tmp_path, "int main() { try { Buffer b; StreamDrain d{(cudaStream_t)%d}; if (%d) throw 1; } catch (int) {} }"
                % (stream, throws))
     assert out == ["sync %d" % stream, "release"]
+
+
+SIDE = r"""
+int main() {
+  const cudaStream_t st = (cudaStream_t)%d, side = (cudaStream_t)2;
+  try {
+    SideScope s(st, side, (cudaEvent_t)11, (cudaEvent_t)12);
+    s.fork();
+    if (%d) throw 1;
+    s.join();
+  } catch (int) {}
+}
+"""
+
+
+@pytest.mark.parametrize("throws", [0, 1])
+def test_side_stream_is_joined(tmp_path, throws):
+    out = _run(tmp_path, SIDE % (1, throws))
+    assert out == ["record 11 on 1", "2 waits for 11", "record 12 on 2", "1 waits for 12"]
+
+
+def test_one_stream_needs_no_events(tmp_path):
+    assert _run(tmp_path, SIDE % (2, 1)) == []
+
+
+def test_builds_fork_through_the_scope():
+    text = open(os.path.join(CSRC, "dfjk_api.cu")).read()
+    build = text[text.index("void build_one("):text.index("// Buffers of the density build")]
+    assert "side.fork()" in build and "cudaStreamWaitEvent" not in build
