@@ -8,6 +8,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <deque>
+#include <initializer_list>
 #include <map>
 #include <mutex>
 #include <string>
@@ -1031,17 +1032,21 @@ void release_device(dfjk_ctx *h) {
   h->resident = false;
 }
 
-// Rows P per chunk of the build: the largest multiple of 128 whose work buffers
-// (X in FP64 and its slices, the slices of B's kept pairs: `steps` K steps of 16
-// over all AOs) stay within DFJK_BUILD_WS_MB megabytes (default 8192), at least
-// 128, at most the whole (padded) aux range.
-int build_chunk_rows(int nao, int np, int nocc, int fmt, long long steps, int ws_mb = 0) {
+// The cap on a build's work buffers.
+size_t build_ws_bytes(int ws_mb) {
   static const size_t cap_env = [] {
     const char *e = std::getenv("DFJK_BUILD_WS_MB");
     const long v = e ? std::atol(e) : 0;
     return (size_t)(v > 0 ? v : 8192) << 20;
   }();
-  const size_t cap = ws_mb > 0 ? (size_t)ws_mb << 20 : cap_env;
+  return ws_mb > 0 ? (size_t)ws_mb << 20 : cap_env;
+}
+// Rows P per chunk of the build: the largest multiple of 128 whose work buffers
+// (X in FP64 and its slices, the slices of B's kept pairs: `steps` K steps of 16
+// over all AOs) stay within DFJK_BUILD_WS_MB megabytes (default 8192), at least
+// 128, at most the whole (padded) aux range.
+int build_chunk_rows(int nao, int np, int nocc, int fmt, long long steps, int ws_mb = 0) {
+  const size_t cap = build_ws_bytes(ws_mb);
   const size_t rp = ((size_t)nao + OZ_BM - 1) / OZ_BM * OZ_BM;
   const size_t el = 2 * (size_t)oz_slices(fmt);  // bytes of an element's slices
   const size_t per_row = (size_t)nao * nocc * 8 + rp * nocc * el + (size_t)steps * OZ_BK * el;
@@ -1816,6 +1821,10 @@ int dfjk_build_density(dfjk_handle h, int32_t nset, const double *D, double *J, 
   }
 }
 
+// Intermediates of a gradient's finished stage up to this size stay to the end of its
+// dense part: giving them back takes a wait of some 20 us.
+constexpr size_t GRAD_HELD_BYTES = (size_t)4 << 30;
+
 // Buffers of a gradient call.
 struct GradWork {
   DBuf<double> D, rho, work, d, X, Xt, Z, stage, W, gam;
@@ -1824,9 +1833,11 @@ struct GradWork {
   DBuf<int> orb_atom, aux_atom, aux_l;
   XWork xw;
   std::deque<SlicedOp> ops;  // slices of the tensor-core GEMMs
-  ~GradWork() {
+  void free_ops() {
     for (SlicedOp &o : ops) oz_free(o);
+    ops.clear();
   }
+  ~GradWork() { free_ops(); }
 };
 
 // d(cj E_J + ck E_K)/dR at fixed D = C C^T (or the given D when ck = 0).
@@ -1880,6 +1891,34 @@ static void jk_gradient(dfjk_ctx *h, const double *Din, int nocc, const double *
     o.status = h->status.p; o.timeout = h->opt.timeout_iters; o.tile_ctr = h->tctr.p;
     oz_gemm(A, Bo, o, st);
   };
+  // out[P][m][n] = sum_k x(P, m, k) B(n, k) for all P, x(P, r, k) = p[P sz + r sr + k sk]: the
+  // slices are cut for ranges of P within a quarter of the build's work-buffer cap
+  auto tc_gemm_per_aux = [&](const double *p, long long sz, long long sr, long long sk, int rows, int K, const SlicedOp &Bo,
+                             int N, double *out, long long ldo, long long obs) {
+    const size_t per = oz_bytes(h->bfmt, rows, K, OZ_BM);
+    const int nb = (int)std::min<size_t>(np, std::max<size_t>(1, build_ws_bytes(h->tune.build_ws_mb) / 4 / per));
+    wk.ops.emplace_back();
+    SlicedOp &o = wk.ops.back();
+    oz_alloc(o, nb, h->bfmt, rows, K, OZ_BM);
+    for (int p0 = 0; p0 < np; p0 += nb) {
+      SlicedOp v = o;
+      v.batch = std::min(nb, np - p0);
+      oz_slice_f64(p + p0 * sz, sz, sr, sk, v, st);
+      tc_gemm(v, Bo, rows, N, K, v.batch, out + p0 * obs, ldo, obs, 0);
+    }
+  };
+  // What a finished stage held goes back once it amounts to something: FP64 slices are
+  // twice their operand's size, and G alone is naux_pad nao^2 doubles.
+  auto stage_done = [&](std::initializer_list<DBuf<double> *> bufs) {
+    size_t held = wk.xw.bsl.bytes() + wk.xw.cdat.bytes();
+    for (const SlicedOp &o : wk.ops) held += o.data_bytes();
+    for (DBuf<double> *b : bufs) held += b->bytes();
+    if (held < GRAD_HELD_BYTES) return;
+    DFJK_CUDA_CHECK(cudaStreamSynchronize(st));
+    for (DBuf<double> *b : bufs) b->release();
+    wk.xw.release();
+    wk.free_ops();
+  };
   if (ck != 0.0) {
     // the build's slices on the tensor cores, or FP64 CUDA-core GEMMs for the small
     // molecules of DFJK_FP64
@@ -1891,10 +1930,8 @@ static void jk_gradient(dfjk_ctx *h, const double *Din, int nocc, const double *
     Xt.alloc((size_t)np * no2);
     Z.alloc((size_t)np * no2);
     W.alloc((size_t)np * np);
-    gam.alloc((size_t)np * nao * nao);
     if (tc) {
       const SlicedOp &csl = slice(C, 0, 1, nocc, 1, nocc, nao, OZ_BN);  // rows i, K nu
-      const SlicedOp &cn = slice(C, 0, nocc, 1, 1, nao, nocc, OZ_BN);   // rows mu, K i
       // X[mu][P][i] = sum_nu B[(mu,nu)][P] C[nu][i], chunk by chunk of rows P
       // as the build does
       const int pcm = build_chunk_rows(nao, np, nocc, h->bfmt, h->pl.steps, h->tune.build_ws_mb);
@@ -1909,8 +1946,8 @@ static void jk_gradient(dfjk_ctx *h, const double *Din, int nocc, const double *
                             (long long)np * nocc, 0, p0 == 0}, st);
       }
       // Xt[P][j][i] = sum_mu X[mu][P][j] C[mu][i]  (symmetric in i, j)
-      const SlicedOp &xs = slice(X.p, nocc, 1, (long long)np * nocc, np, nocc, nao, OZ_BM);
-      tc_gemm(xs, csl, nocc, nocc, nao, np, Xt.p, nocc, no2, 0);
+      tc_gemm_per_aux(X.p, nocc, 1, (long long)np * nocc, nocc, nao, csl, nocc, Xt.p, nocc, no2);
+      stage_done({&stage});
       // Z[P][ij] = sum_Q Linv[Q][P] Xt[Q][ij]
       const SlicedOp &lt = slice(h->Linv.p, 0, 1, np, 1, np, np, OZ_BM);
       const SlicedOp &xts = slice(Xt.p, 0, 1, no2, 1, (int)no2, np, OZ_BN);
@@ -1920,12 +1957,14 @@ static void jk_gradient(dfjk_ctx *h, const double *Din, int nocc, const double *
       tc_gemm(zs, zs, np, np, (int)no2, 1, W.p, np, 0, 1);
       mirror_lower_f64(W.p, np, st);
       // Yt[P][j][mu] = sum_i Z[P][i][j] C[mu][i]   (Yt reuses X)
-      const SlicedOp &zb = slice(Z.p, no2, 1, nocc, np, nocc, nocc, OZ_BM);
-      tc_gemm(zb, cn, nocc, nao, nocc, np, X.p, nao, (long long)nao * nocc, 0);
+      stage_done({&Xt});
+      const SlicedOp &cn = slice(C, 0, nocc, 1, 1, nao, nocc, OZ_BN);  // rows mu, K i
+      tc_gemm_per_aux(Z.p, no2, 1, nocc, nocc, nocc, cn, nao, X.p, nao, (long long)nao * nocc);
       // Gam[P][mu][nu] = sum_j Yt[P][j][mu] C[nu][j]
-      const SlicedOp &ys = slice(X.p, (long long)nao * nocc, 1, nao, np, nao, nocc, OZ_BM);
-      tc_gemm(ys, cn, nao, nao, nocc, np, gam.p, nao, (long long)nao * nao, 0);
+      gam.alloc((size_t)np * nao * nao);
+      tc_gemm_per_aux(X.p, (long long)nao * nocc, 1, nao, nao, nocc, cn, nao, gam.p, nao, (long long)nao * nao);
     } else {
+      gam.alloc((size_t)np * nao * nao);
       GemmArgs x;  // X[mu][P][i] = sum_nu B[(mu,nu)][P] C[nu][i]
       x.M = np; x.N = nocc; x.K = nao; x.batch = nao;
       x.A = h->B.p; x.sAm = 1; x.sAk = h->ldb; x.sAb = (long long)nao * h->ldb;
@@ -1968,6 +2007,7 @@ static void jk_gradient(dfjk_ctx *h, const double *Din, int nocc, const double *
     DFJK_CUDA_CHECK(cudaStreamSynchronize(st));
     for (DBuf<double> *b : {&X, &Xt, &Z, &stage}) b->release();
     xw.release();
+    wk.free_ops();
   }
   DBuf<int> &oat = wk.orb_atom, &aat = wk.aux_atom, &al = wk.aux_l;
   oat.upload(h->orb.atom, st);

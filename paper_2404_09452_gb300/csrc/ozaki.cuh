@@ -53,6 +53,8 @@ struct SlicedOp {
 // Sizes an operand (rows padded to `row_tile`, K to OZ_BK) and allocates it.
 void oz_alloc(SlicedOp &op, int batch, int fmt, int rows, int K, int row_tile);
 void oz_free(SlicedOp &op);
+// Bytes of the slices of one batch of such an operand.
+size_t oz_bytes(int fmt, int rows, int K, int row_tile);
 // A view of op's buffers sized for `rows` rows and K columns (at most the
 // allocated rows and K): the layout a fresh allocation of that size would
 // have, placed at the start of op's buffers.  Used for the short last chunk

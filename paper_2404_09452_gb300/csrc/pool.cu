@@ -28,12 +28,17 @@ struct DevCache {
   std::map<uint64_t, std::multimap<size_t, Block>::iterator> by_time;      // oldest first
   std::unordered_map<void *, size_t> size_of;                              // every block handed out or cached
   size_t bytes = 0;
+  size_t used = 0, peak = 0;  // bytes handed out, and the most since dfjk_debug_pool_peak
   uint64_t clock = 0;
 
   std::multimap<size_t, Block>::iterator take(std::multimap<size_t, Block>::iterator it) {
     by_time.erase(it->second.when);
     bytes -= it->first;
     return blocks.erase(it);
+  }
+  void hand_out(size_t b) {
+    used += b;
+    peak = peak > used ? peak : used;
   }
   void drop_oldest() {
     auto it = by_time.begin()->second;
@@ -74,6 +79,7 @@ void *pool_alloc(size_t bytes) {
     auto it = c.blocks.lower_bound(bytes);
     if (it != c.blocks.end() && it->first <= bytes + bytes / 8) {
       void *p = it->second.p;
+      c.hand_out(it->first);
       c.take(it);
       return p;
     }
@@ -94,6 +100,7 @@ void *pool_alloc(size_t bytes) {
   }
   std::lock_guard<std::mutex> lk(g_mu);
   g_cache[dev].size_of[p] = bytes;
+  g_cache[dev].hand_out(bytes);
   return p;
 }
 
@@ -107,6 +114,7 @@ void pool_free(void *p, size_t) {
   std::lock_guard<std::mutex> lk(g_mu);
   DevCache &c = g_cache[dev];
   const auto known = c.size_of.find(p);
+  if (known != c.size_of.end()) c.used -= known->second;
   if (known == c.size_of.end() || known->second > cache_limit()) {
     if (known != c.size_of.end()) c.size_of.erase(known);
     cudaFree(p);
@@ -132,6 +140,20 @@ size_t pool_cached_bytes() {
 }
 
 }  // namespace dfjk
+
+// For tests: the most bytes handed out at a time on this device since the last call.
+extern "C" size_t dfjk_debug_pool_peak(void) {
+  try {
+    const int dev = dfjk::current_device();
+    std::lock_guard<std::mutex> lk(dfjk::g_mu);
+    dfjk::DevCache &c = dfjk::g_cache[dev];
+    const size_t peak = c.peak;
+    c.peak = c.used;
+    return peak;
+  } catch (const dfjk::Error &) {
+    return 0;
+  }
+}
 
 extern "C" int dfjk_trim_cache(void) {
   try {
