@@ -1831,6 +1831,7 @@ struct GradWork {
   DBuf<double> rec, gm;  // pair records and weights: doubles or double-single pairs
   DBuf<long long> goff;
   DBuf<int> orb_atom, aux_atom, aux_l;
+  DBuf<unsigned> top;  // high words of the largest |D|, |d|, |C|, |Z|
   XWork xw;
   std::deque<SlicedOp> ops;  // slices of the tensor-core GEMMs
   void free_ops() {
@@ -1839,6 +1840,12 @@ struct GradWork {
   }
   ~GradWork() { free_ops(); }
 };
+
+// Whether weights of this size keep the double-single derivative kernels inside the FP32
+// range: they multiply Hermite integrals of up to 1e28 (exponents of 1e4) on the way
+// up and lose the low parts near 1e-38 on the way down.  Densities far from 1 (scaled
+// or difference densities) take the FP64 kernels.
+static bool df_weight_ok(double w, double lo, double hi) { return w == 0.0 || (w >= lo && w <= hi); }
 
 // d(cj E_J + ck E_K)/dR at fixed D = C C^T (or the given D when ck = 0).
 // E = sum_PQ (V^-1)_PQ M_PQ / 2 for both energies, M_PQ = u_P u_Q (J) or
@@ -1919,7 +1926,12 @@ static void jk_gradient(dfjk_ctx *h, const double *Din, int nocc, const double *
     wk.xw.release();
     wk.free_ops();
   };
-  if (ck != 0.0) {
+  const bool exch = ck != 0.0;
+  AbsMax am{};
+  am.x[0] = D; am.n[0] = (long long)nao * nao;
+  am.x[1] = d.p; am.n[1] = h->naux;
+  wk.top.alloc(4);
+  if (exch) {
     // the build's slices on the tensor cores, or FP64 CUDA-core GEMMs for the small
     // molecules of DFJK_FP64
     const bool tc = h->sliced;
@@ -2004,23 +2016,26 @@ static void jk_gradient(dfjk_ctx *h, const double *Din, int nocc, const double *
       gm.C = gam.p; gm.sCm = nao; gm.sCn = 1; gm.sCb = (long long)nao * nao;
       gemm_f64(gm, st);
     }
+    am.x[2] = C; am.n[2] = (long long)nao * nocc;
+    am.x[3] = Z.p; am.n[3] = np * no2;
+  }
+  if (h->use_df) abs_max(am, wk.top.p, st);
+  if (exch) {
     DFJK_CUDA_CHECK(cudaStreamSynchronize(st));
-    for (DBuf<double> *b : {&X, &Xt, &Z, &stage}) b->release();
-    xw.release();
+    for (DBuf<double> *b : {&wk.X, &wk.Xt, &wk.Z, &wk.stage}) b->release();
+    wk.xw.release();
     wk.free_ops();
   }
   DBuf<int> &oat = wk.orb_atom, &aat = wk.aux_atom, &al = wk.aux_l;
   oat.upload(h->orb.atom, st);
   aat.upload(h->aux.atom, st);
   al.upload(h->aux.l, st);
-  DFJK_CUDA_CHECK(cudaMemsetAsync(grad, 0, sizeof(double) * 3 * (size_t)h->natom, st));
   GradArgs g{};
   g.pair_a = h->pair_a.p;
   g.pair_b = h->pair_b.p;
   g.npp = h->pair_npp.p;
   g.pair_col = h->pair_col.p;
   g.ldg = np;
-  for (int q = 0; q < 3; ++q) g.c0[q] = h->use_df ? h->c0[q] : 0.0;
   g.d = d.p;
   g.D = D;
   g.nao = nao;
@@ -2033,11 +2048,6 @@ static void jk_gradient(dfjk_ctx *h, const double *Din, int nocc, const double *
   g.aux_atom = aat.p;
   g.grad = grad;
   static const int cls[6][2] = {{0, 0}, {1, 0}, {1, 1}, {2, 0}, {2, 1}, {2, 2}};
-  // Coulomb-only gradients of a mixed handle take the build's precision split: the
-  // kept pairs it evaluates in FP32 (Schwarz bound below fp32_pair_thresh) get FP32
-  // derivative weights, the others double-single (FP64 beyond its range)
-  const bool exch = ck != 0.0, dfs = h->use_df;
-  const bool split32 = !exch && dfs;
   const GradBoysTabs tabs{tab, boys_table_device_f32(), boys_table_device_df()};
   std::vector<long long> off(h->npair_kept + 1, 0);
   for (int c = 0; c < 6; ++c)
@@ -2048,41 +2058,62 @@ static void jk_gradient(dfjk_ctx *h, const double *Din, int nocc, const double *
   DBuf<double> &rec = wk.rec, &gm = wk.gm;
   rec.alloc(std::max<size_t>(1, (size_t)off.back()));
   if (exch) gm.alloc((size_t)std::max<long long>(h->ncol, 1) * np);
-  for (int c = 0; c < 6; ++c) {
-    g.pairs = h->kept.p + h->kept_cls_begin[c];
-    g.npairs = h->kept_cls_begin[c + 1] - h->kept_cls_begin[c];
-    g.rec_off = goff.p + h->kept_cls_begin[c];
-    launch_grad_tables(cls[c][0], cls[c][1], exch, dfs, g, orb_args(h), rec.p, st);
-    if (exch) launch_grad_gamma(cls[c][0], cls[c][1], dfs, g, orb_args(h), h->naux, gm.p, st);
-  }
-  g.rec = rec.p;
-  g.gamma = gm.p;
-  // The classes run on the integral streams, the largest first: one after the other each
-  // left the GPU to its own last wave: 45 atoms (Coulomb) 11.3 -> 9.7 ms,
-  // 30 atoms (Coulomb and exchange) 19.2 -> 16.1.
-  {
-    const IntegralFork fork(st, h->ev_int);
-    launch_grad2c(g, aux_args(h), al.p, h->aux.nshell, tab, fork.is[INT_STREAMS - 1]);
-    for (int c = 5; c >= 0; --c) {
-      const int lo = h->kept_cls_begin[c], hi = h->kept_cls_begin[c + 1];
-      if (hi <= lo) continue;
-      const int mid = split32 ? std::min(std::max(lo, h->kept32_begin[c]), hi) : hi;
-      for (int lc = 2; lc >= 0; --lc) {
-        g.aux_shells = h->aux_cls[lc].p;
-        g.naux_shells = h->aux_cls_n[lc];
-        g.pairs = h->kept.p + lo;
-        g.rec_off = goff.p + lo;
-        g.npairs = mid - lo;
-        launch_grad3c(cls[c][0], cls[c][1], lc, dfs ? GRAD_DF : GRAD_F64, g, aux_args(h), tabs,
-                      fork.is[(c + lc) % (INT_STREAMS - 1)]);
-        g.pairs = h->kept.p + mid;
-        g.rec_off = goff.p + mid;
-        g.npairs = hi - mid;
-        launch_grad3c(cls[c][0], cls[c][1], lc, GRAD_F32, g, aux_args(h), tabs, fork.is[INT_STREAMS - 1]);
+  const auto run = [&](bool dfs) {
+    DFJK_CUDA_CHECK(cudaMemsetAsync(grad, 0, sizeof(double) * 3 * (size_t)h->natom, st));
+    // Coulomb-only gradients of a mixed handle take the build's precision split: the
+    // kept pairs it evaluates in FP32 (Schwarz bound below fp32_pair_thresh) get FP32
+    // derivative weights, the others double-single (FP64 beyond its range)
+    const bool split32 = !exch && dfs;
+    for (int q = 0; q < 3; ++q) g.c0[q] = dfs ? h->c0[q] : 0.0;
+    for (int c = 0; c < 6; ++c) {
+      g.pairs = h->kept.p + h->kept_cls_begin[c];
+      g.npairs = h->kept_cls_begin[c + 1] - h->kept_cls_begin[c];
+      g.rec_off = goff.p + h->kept_cls_begin[c];
+      launch_grad_tables(cls[c][0], cls[c][1], exch, dfs, g, orb_args(h), rec.p, st);
+      if (exch) launch_grad_gamma(cls[c][0], cls[c][1], dfs, g, orb_args(h), h->naux, gm.p, st);
+    }
+    g.rec = rec.p;
+    g.gamma = gm.p;
+    // The classes run on the integral streams, the largest first: one after the other each
+    // left the GPU to its own last wave: 45 atoms (Coulomb) 11.3 -> 9.7 ms,
+    // 30 atoms (Coulomb and exchange) 19.2 -> 16.1.
+    {
+      const IntegralFork fork(st, h->ev_int);
+      launch_grad2c(g, aux_args(h), al.p, h->aux.nshell, tab, fork.is[INT_STREAMS - 1]);
+      for (int c = 5; c >= 0; --c) {
+        const int lo = h->kept_cls_begin[c], hi = h->kept_cls_begin[c + 1];
+        if (hi <= lo) continue;
+        const int mid = split32 ? std::min(std::max(lo, h->kept32_begin[c]), hi) : hi;
+        for (int lc = 2; lc >= 0; --lc) {
+          g.aux_shells = h->aux_cls[lc].p;
+          g.naux_shells = h->aux_cls_n[lc];
+          g.pairs = h->kept.p + lo;
+          g.rec_off = goff.p + lo;
+          g.npairs = mid - lo;
+          launch_grad3c(cls[c][0], cls[c][1], lc, dfs ? GRAD_DF : GRAD_F64, g, aux_args(h), tabs,
+                        fork.is[(c + lc) % (INT_STREAMS - 1)]);
+          g.pairs = h->kept.p + mid;
+          g.rec_off = goff.p + mid;
+          g.npairs = hi - mid;
+          launch_grad3c(cls[c][0], cls[c][1], lc, GRAD_F32, g, aux_args(h), tabs, fork.is[INT_STREAMS - 1]);
+        }
       }
     }
-  }
+  };
+  run(h->use_df);
+  unsigned top[4] = {0, 0, 0, 0};
+  if (h->use_df) DFJK_CUDA_CHECK(cudaMemcpyAsync(top, wk.top.p, sizeof(top), cudaMemcpyDeviceToHost, st));
   DFJK_CUDA_CHECK(cudaStreamSynchronize(st));
+  if (h->use_df) {
+    const double Dm = abs_max_value(top[0]), dm = std::fabs(cj) * abs_max_value(top[1]), Cm = abs_max_value(top[2]);
+    const double gamma = std::fabs(ck) * Cm * Cm * abs_max_value(top[3]);  // Gam = C Z C^T
+    const bool ok = exch ? df_weight_ok(std::max(dm * Dm, gamma * nocc * nocc), 0x1p-50, 0x1p60)
+                         : df_weight_ok(Dm, 0x1p-40, 0x1p30) && df_weight_ok(dm, 0x1p-40, 0x1p30);
+    if (!ok) {  // once more, in FP64: the rare case pays, not every call with a wait for the sizes
+      run(false);
+      DFJK_CUDA_CHECK(cudaStreamSynchronize(st));
+    }
+  }
   throw_on_timeout(h, "gradient");
 }
 

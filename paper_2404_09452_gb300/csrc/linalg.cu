@@ -10,6 +10,7 @@
 // at any reasonable tiling; they are the plain-FP64 reference path.
 #include <algorithm>
 #include <cmath>
+#include <cstring>
 
 #include "common.cuh"
 #include "linalg.cuh"
@@ -663,6 +664,33 @@ void screen_pairs(const double *q, int n, const double *maxdiag, double thresh, 
   if (n == 0) return;
   screen_kernel<<<ceil_div(n, 256), 256, 0, st>>>(q, n, maxdiag, thresh, keep);
   DFJK_LAUNCHED();
+}
+
+// Non-negative doubles order like their bits, so the maxima are of 32-bit integers (the
+// FP64 pipe is the scarce one); bound by reading the arrays.
+__global__ void __launch_bounds__(256) abs_max_kernel(AbsMax a, unsigned *out) {
+  const double *x = a.x[blockIdx.y];
+  const long long n = a.n[blockIdx.y];
+  unsigned m = 0;
+  for (long long i = (long long)blockIdx.x * 256 + threadIdx.x; i < n; i += (long long)gridDim.x * 256)
+    m = max(m, (unsigned)__double2hiint(x[i]) & 0x7FFFFFFFu);
+  m = __reduce_max_sync(0xffffffffu, m);
+  if ((threadIdx.x & 31) == 0 && m > 0) atomicMax(out + blockIdx.y, m);
+}
+
+void abs_max(const AbsMax &a, unsigned *out, cudaStream_t st) {
+  long long most = 1;
+  for (long long n : a.n) most = std::max(most, n);
+  DFJK_CUDA_CHECK(cudaMemsetAsync(out, 0, 4 * sizeof(unsigned), st));
+  abs_max_kernel<<<dim3((unsigned)std::min<long long>((most + 255) / 256, 152 * 8), 4), 256, 0, st>>>(a, out);
+  DFJK_LAUNCHED();
+}
+
+double abs_max_value(unsigned hi) {
+  const uint64_t u = (uint64_t)hi << 32;
+  double v;
+  std::memcpy(&v, &u, sizeof(v));
+  return v;
 }
 
 __global__ void fill_kernel(double *p, long long n, double v) {

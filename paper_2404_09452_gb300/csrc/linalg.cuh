@@ -87,6 +87,14 @@ void max_sqrt_diag(const double *V, int n, int ld, double *out, cudaStream_t st)
 // keep[i] = q[i] * (*maxdiag) >= thresh
 void screen_pairs(const double *q, int n, const double *maxdiag, double thresh, int *keep,
                   cudaStream_t st);
+// out[i] = high word of the largest |x_i| of n[i] elements (0 for none), for up to four arrays
+// at once; abs_max_value: that element to within its low word (infinities and NaN as such).
+struct AbsMax {
+  const double *x[4];
+  long long n[4];
+};
+void abs_max(const AbsMax &a, unsigned *out, cudaStream_t st);
+double abs_max_value(unsigned hi);
 void fill_f64(double *p, long long n, double v, cudaStream_t st);
 // out[i][j] = in[perm_r[i] * ldi + perm_c[j]] for an n_r x n_c gather (0 where
 // perm_r[i] < 0).
