@@ -389,10 +389,11 @@ int dfjk_get_B_columns(dfjk_handle h, int32_t ncol, const int32_t *mu, const int
  * naux x nao x nao; recomputed on demand.                                    */
 int dfjk_get_three_center(dfjk_handle h, double *T, void *stream);
 
-/* The exact sliced-product tensor-core GEMM used by DFJK_MIXED, on its own:
+/* The exact sliced-product tensor-core GEMM, on its own:
  * C[z][m][n] = sum_k A[z][m][k] B[n][k] with A (batch x M x K), B (N x K),
- * C (batch x M x N) device FP64 row-major; S = 6 or 8 slices of 6 bits per
- * operand row and 1024-wide K block.  Allocates its slice buffers, synchronises
+ * C (batch x M x N) device FP64 row-major; S = 6 or 8: slices of 6 bits per
+ * operand row and 1024-wide K block (DFJK_MIXED); S = 56: the 8 slices of 7 bits
+ * and 384-wide K blocks of DFJK_FP64.  Allocates its slice buffers, synchronises
  * `stream`.  *status (device int, may be NULL) receives STATUS bits.         */
 int dfjk_debug_sliced_gemm(int32_t batch, int32_t M, int32_t N, int32_t K, int32_t S,
                            const double *A, const double *B, double *C, int32_t *status,

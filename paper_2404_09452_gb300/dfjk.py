@@ -488,7 +488,8 @@ def phase_times() -> dict:
 
 def sliced_gemm(A, B, S=6, stream=None):
     """C[z] = A[z] B^T through the exact sliced tensor-core GEMM (FP64 device
-    tensors; A [batch, M, K] or [M, K], B [N, K])."""
+    tensors; A [batch, M, K] or [M, K], B [N, K]); S = 6 or 8 slices of 6 bits,
+    or 56 for the FP64 path's 56 bits."""
     torch = _torch()
     A3 = A.contiguous().reshape(-1, A.shape[-2], A.shape[-1])
     B = B.contiguous()
