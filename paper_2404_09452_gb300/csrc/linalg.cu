@@ -693,18 +693,6 @@ double abs_max_value(unsigned hi) {
   return v;
 }
 
-__global__ void fill_kernel(double *p, long long n, double v) {
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (long long)gridDim.x * blockDim.x)
-    p[i] = v;
-}
-
-void fill_f64(double *p, long long n, double v, cudaStream_t st) {
-  if (n == 0) return;
-  fill_kernel<<<(unsigned)std::min<long long>((n + 255) / 256, 4096), 256, 0, st>>>(p, n, v);
-  DFJK_LAUNCHED();
-}
-
 __global__ void gather2d_kernel(const double *in, long long ldi, const int *pr, const int *pc,
                                 int nr, int nc, double *out, long long ldo) {
   const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;

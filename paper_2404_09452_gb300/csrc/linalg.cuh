@@ -50,9 +50,6 @@ struct CholStreams {
 };
 void cholesky_inverse_f64(double *A, int n, int lda, double *Dinv, double *Linv, double *work, int *status,
                           const CholStreams &cs);
-// cholesky_f64 and `work` (n x n doubles).
-void tri_inverse_f64(const double *L, int n, int ld, const double *Dinv, double *Linv,
-                     double *work, cudaStream_t st);
 
 // Both triangles of a row-mapped B: Bfull[(mu nao + nu) ldb + P] (nao^2 rows).
 void unpack_rows_f64(const double *Bc, long long ldb, int nao, const int *rowmap, double *Bfull, cudaStream_t st);
@@ -95,7 +92,6 @@ struct AbsMax {
 };
 void abs_max(const AbsMax &a, unsigned *out, cudaStream_t st);
 double abs_max_value(unsigned hi);
-void fill_f64(double *p, long long n, double v, cudaStream_t st);
 // out[i][j] = in[perm_r[i] * ldi + perm_c[j]] for an n_r x n_c gather (0 where
 // perm_r[i] < 0).
 void gather2d_f64(const double *in, long long ldi, const int *perm_r, const int *perm_c, int nr,
