@@ -46,7 +46,7 @@ PAIR_CLASSES = [(0, 0), (1, 0), (1, 1), (2, 0), (2, 1), (2, 2)]
 
 def eri_flops_per_triple():
     """FP64 and FP32 flops per primitive triple of each 3-centre integral
-    kernel, {(LA, LB, LC, "fp64"|"fp32"): (dflop, sflop)}: the ncu instruction
+    kernel, {(LA, LB, LC, "fp64"|"df"|"fp32"): (dflop, sflop)}: the ncu instruction
     counts of one capture (DFMA x2 + DMUL + DADD; FFMA x2 + FFMA2 x4 + FMUL +
     FADD) divided by the primitive triples that launch processed, both
     recorded in profiles/eri3c_mol20.md; empty when the kernel source
@@ -60,22 +60,24 @@ def eri_flops_per_triple():
     out = {}
     for line in open(ERI_COUNTS_FILE):
         f = line.split()
-        # eri3c-count <LA> <LB> <LC> <fp64|fp32> <primitive triples> <dflop> <sflop> <sha16 of md.cuh>
+        # eri3c-count <LA> <LB> <LC> <fp64|df|fp32> <primitive triples> <dflop> <sflop> <sha16 of md.cuh>
         if len(f) == 9 and f[0] == "eri3c-count" and f[8] == sha and int(f[5]) > 0:
             n = float(f[5])
             out[(int(f[1]), int(f[2]), int(f[3]), f[4])] = (float(f[6]) / n, float(f[7]) / n)
     return out
 
 
-def eri_roofline(h, m, ms64, ms32, fp64_peak, fp32_peak):
-    """Roofline of the 3-centre integral phase (FP64-ALU bound): counted
+def eri_roofline(h, m, ms64, ms32, fp64_peak, fp32_peak, big="fp64"):
+    """Roofline of the 3-centre integral phase (ALU bound): counted
     flops of the step's primitive triples per precision, divided by the
-    phase's CUDA-event time, against the measured FMA rates."""
+    phase's CUDA-event time, against the measured FMA rates.  `big`: arithmetic
+    of the pairs above the FP32 threshold; double-single ("df") runs on the FP32
+    pipe, beside the FP32 pairs and within the same span ms64."""
     per = eri_flops_per_triple()
     if not per:
         return None
     naux_prims = [sum(len(sh.exps) for sh in m.aux.shells if sh.l == lc) for lc in range(3)]
-    f64 = f32_s = f32_d = 0.0
+    f64 = f32_s = f32_d = df_s = 0.0
     trip64 = trip32 = 0
     for c, (la, lb) in enumerate(PAIR_CLASSES):
         for lc in range(3):
@@ -83,14 +85,21 @@ def eri_roofline(h, m, ms64, ms32, fp64_peak, fp32_peak):
             t32 = h.prim_pairs_fp32[c] * naux_prims[lc]
             trip64 += t64
             trip32 += t32
-            d, _ = per.get((la, lb, lc, "fp64"), (0.0, 0.0))
+            d, s = per.get((la, lb, lc, big), (0.0, 0.0))
             d32, s32 = per.get((la, lb, lc, "fp32"), (0.0, 0.0))
             f64 += t64 * d
+            df_s += t64 * s
             f32_d += t32 * d32
             f32_s += t32 * s32
-    out = {"bound": "alu", "unit": "TFLOP/s", "primitive_triples_fp64": trip64,
+    out = {"bound": "alu", "unit": "TFLOP/s", f"primitive_triples_{big}": trip64,
            "primitive_triples_fp32": trip32, "flop_source": "ncu instruction counts per primitive triple "
            "(profiles/eri3c_mol20.md)"}
+    if big == "df":
+        if ms64:
+            a = (df_s + f32_s) / (ms64 / 1e3) / 1e12
+            out["fp32"] = {"flops": df_s + f32_s, "of_fp32_pairs": f32_s, "ms": ms64, "achieved": a, "peak": fp32_peak,
+                           "frac": a / fp32_peak, "peak_source": "dfjk_fma_rate(32), measured in this run"}
+        return out
     if ms64:
         a = f64 / (ms64 / 1e3) / 1e12
         out["fp64"] = {"flops": f64, "ms": ms64, "achieved": a, "peak": fp64_peak, "frac": a / fp64_peak,
@@ -497,15 +506,19 @@ def run_ours(args):
             dist.destroy_process_group()
         return
 
+    fp64 = prec == dfjk.DFJK_FP64
+    np_pad = (m.naux + 63) // 64 * 64
+    sliced = not fp64 or m.nao * m.nao * np_pad >= 3e5  # dense products on the tensor cores
     flops = algorithmic_flops(m.nao, m.naux, nocc, ncol)
+    kept = (2 * int(ncol) - m.nao) / m.nao**2 if sliced else 1.0  # X runs over the kept pairs, in both orders
+    flops["X=BC"] *= kept
     per_step = {k: v / args.steps for k, v in phases.items()}
     step_flops = sum(flops.values())
-    fp64 = prec == dfjk.DFJK_FP64
     peaks = {}
     if os.path.exists(PEAKS_FILE):
         peaks = json.load(open(PEAKS_FILE))
     bf16_sust = float(peaks.get("bf16_tflops_sustained", 1700.0))
-    if fp64:
+    if not sliced:
         dom = max(flops, key=lambda k: per_step.get(k, 0.0))
         dom_ms = per_step[dom]
         achieved = flops[dom] / (dom_ms / 1e3) / 1e12
@@ -517,38 +530,40 @@ def run_ours(args):
     else:
         # tensor-core GEMM launches alone; products = exact slice products per
         # FP64-equivalent multiply-add (S (S+1) / 2 with S = 8 or 6 slices)
-        tc = {"whiten": ("tc:whiten", 36), "X=BC": ("tc:X=BC", 21), "K": ("tc:K", 21)}
+        xk = 36 if fp64 else 21
+        tc = {"whiten": ("tc:whiten", 36), "X=BC": ("tc:X=BC", xk), "K": ("tc:K", xk)}
         dom = max(tc, key=lambda k: per_step.get(tc[k][0], 0.0))
         key, prods = tc[dom]
-        # launches per step: whitening one per T slab, X and K one per aux chunk
+        # launches per step: whitening one per T slab, X and K one per aux chunk (FP64
+        # handles do not report theirs: all of a step's launches together)
         nl = nslab if dom == "whiten" else max(1, chunks[1])
         dom_ms = per_step[key] / nl
         achieved = flops[dom] / nl / (dom_ms / 1e3) / 1e12
-        roof = {"kernel": "oz_gemm_kernel (" + dom + ")", "bound": "tensor", "achieved": achieved,
+        gemm_bytes = algorithmic_bytes(m.nao, m.naux, nocc, ncol)
+        gemm_bytes["X=BC"] -= 12.0 * (1.0 - kept) * m.nao * m.nao * np_pad
+        roof = {"kernel": "oz_gemm_ws_kernel (" + dom + ")", "bound": "tensor", "achieved": achieved,
                 "unit": "TFLOP/s", "peak": bf16_sust / prods,
                 "peak_source": f"measured sustained BF16 dense {bf16_sust} TFLOP/s of measured "
                                f"(MEASURED_PEAKS.json) / {prods} exact slice products",
                 "tensor_pipe_tflops": achieved * prods, "traffic": recorded_traffic(dom, args.workload),
                 "algorithmic_flops_per_launch": flops[dom] / nl, "ms_per_launch": dom_ms,
-                "algorithmic_bytes_per_launch": algorithmic_bytes(m.nao, m.naux, nocc, ncol)[dom] / nl,
+                "algorithmic_bytes_per_launch": None if fp64 else gemm_bytes[dom] / nl,
                 "launches_per_step": nl}
     roof["frac"] = roof["achieved"] / roof["peak"]
     # per-row units of the measurement table: a4 as shell triples/s and
-    # integrals/s, a8 (rho from X, then J over the rows of B: the kept
-    # columns in the mixed path, the mu >= nu rows in FP64) as GB/s
+    # integrals/s, a8 (rho and J, each over the kept rows of B; FP64 handles of a few
+    # atoms: rho from X, then J over the mu >= nu rows) as GB/s
     triples = int(fp32_pairs["kept_shell_pairs"]) * len(m.aux.shells)
     n_int = int(ncol) * int(m.naux)
     eri_ms = per_step.get("eri3c", 0.0)  # spans the FP32 classes too (eri3c32), which run beside the others
-    np_pad = (m.naux + 63) // 64 * 64
-    b_rows = m.nao * (m.nao + 1) // 2 if fp64 else int(ncol)
-    j_bytes = (b_rows * np_pad + m.nao * np_pad * nocc) * 8
+    j_bytes = 2 * int(ncol) * np_pad * 8 if sliced else (m.nao * (m.nao + 1) // 2 + m.nao * nocc) * np_pad * 8
     j_ms = per_step.get("rho+J", 0.0)
     units = {"a4_integrals": {"shell_triples": triples, "integrals": n_int, "ms": eri_ms,
                               "shell_triples_per_s": triples / (eri_ms / 1e3) if eri_ms else None,
                               "integrals_per_s": n_int / (eri_ms / 1e3) if eri_ms else None},
              "a8_rho_J": {"bytes": j_bytes, "ms": j_ms,
                           "GB_per_s": j_bytes / (j_ms / 1e3) / 1e9 if j_ms else None,
-                          "note": "side stream, beside the K GEMM"}}
+                          "note": "side stream, beside the slicing and GEMMs" if sliced else "between X and K"}}
     out = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": total_ms / args.steps, "higher_is_better": True,
@@ -568,7 +583,7 @@ def run_ours(args):
         "roofline": roof,
         "units": units,
         "roofline_a4": eri_roofline(pair_work, m, per_step.get("eri3c", 0.0), per_step.get("eri3c32", 0.0),
-                                    fp64_peak, fp32_peak),
+                                    fp64_peak, fp32_peak, "fp64" if fp64 or args.fp32_pair_thresh == 0 else "df"),
         "fma_peaks_tflops": {"fp64": fp64_peak, "fp32": fp32_peak},
         "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": int(h2d),
                 "d2h_bytes_per_step": int(d2h)},

@@ -76,23 +76,27 @@ typedef struct {
  * tensor cores); DFJK_MIXED does the same for the three dense contractions
  * while keeping FP64-level results.                                          */
 typedef enum {
-  DFJK_FP64 = 0, /* FP64 throughout.  The dense products (whitening, X = B C,
-                    K, the gradient's and the density build's) run on the
-                    tensor cores as exact products of 8 slices of 7 bits, 56
-                    bits below a row's largest element per 384-element block
-                    and dropped terms below 2^-57, recombined in FP64 (errors
-                    against 64-bit references equal the FP64 pipe's); small
-                    molecules (nao^2 naux below 3e5) take the FP64 pipe.  B is
-                    kept in both triangles, nao^2 naux_pad doubles            */
+  DFJK_FP64 = 0, /* FP64, with the dense products (whitening, X = B C, K, the
+                    gradient's and the density build's) on the tensor cores
+                    as exact products of 8 slices of 7 bits, recombined in
+                    FP64: an operand keeps 56 bits below the largest element
+                    of its row and 384-element block (so an element far below
+                    that one keeps fewer than FP64's 53), and slice products
+                    below 2^-57 of the two largest are dropped.  J, K and
+                    gradients are as far from 64-bit references as with FP64
+                    multiply-adds, 1e-13 to 1e-11 of the largest element by
+                    the metric's condition.  Small molecules (nao^2 naux below
+                    3e5) take the FP64 pipe.  B is kept in both triangles,
+                    nao^2 naux_pad doubles                                    */
   DFJK_MIXED = 1 /* 3-centre integrals and their derivatives in
                     double-single arithmetic (two FP32 numbers, about 48 bits;
                     FP64 for exponents outside 1e-4 .. 1e4, atoms more than
                     256 bohr from the centroid or fp32_pair_thresh = 0; FP32
-                    for the pairs below fp32_pair_thresh), the metric, Cholesky and inverse, rho, J
-                    and the energies in FP64.  B is kept in FP64 for the
-                    Schwarz-kept AO pairs only, one row of naux_pad doubles
-                    per kept column (a quarter of the mu >= nu pairs at 60
-                    atoms, fewer for larger molecules).
+                    for the pairs below fp32_pair_thresh), the metric,
+                    Cholesky and inverse, rho, J and the energies in FP64.  B
+                    is kept in FP64 for the Schwarz-kept AO pairs only, one
+                    row of naux_pad doubles per kept column (a quarter of the
+                    mu >= nu pairs at 60 atoms, fewer for larger molecules).
                     The whitening, X = B C and K run on the tensor cores as
                     exact sliced products: each FP64 operand row is cut into 6
                     (8 for the whitening) 6-bit integer slices stored as BF16
@@ -134,9 +138,9 @@ typedef struct {
                               memory                                        */
   const char *tune_table;  /* path of a tuning table (written by the
                               package's autotuner, tune.py): per range of
-                              nao, rows per block of the slicing kernels, the
-                              K GEMM's split-K range and the mixed build's
-                              work-buffer cap; read during dfjk_setup (not
+                              nao, rows (for B, warps) per block of the slicing
+                              kernels, the K GEMM's split-K range and the
+                              build's work-buffer cap; read during dfjk_setup (not
                               kept).  NULL: the DFJK_TUNE_TABLE environment
                               variable, else built-in defaults.  These only
                               change launch shapes: the slicing choices leave
@@ -173,31 +177,34 @@ int dfjk_query(dfjk_handle h, int32_t *nao, int32_t *naux, int32_t *npair_kept,
 
 /* Precision split of the 3-centre integrals of a handle: the number of kept
  * shell pairs evaluated in FP32 and the bound threshold that selected them
- * (0 when every pair is FP64).  Either output pointer may be NULL.           */
+ * (0: none).  Either output pointer may be NULL.                            */
 int dfjk_query_precision(dfjk_handle h, int32_t *npair_fp32, double *fp32_thresh);
 
 /* Work of a handle's 3-centre integrals: the kept primitive pairs of each
- * orbital shell-pair class (ss, ps, pp, ds, dp, dd), evaluated in FP64
- * (prim_pairs_fp64[6]) and in FP32 (prim_pairs_fp32[6]).  Each meets every
+ * orbital shell-pair class (ss, ps, pp, ds, dp, dd), evaluated in FP32
+ * (prim_pairs_fp32[6]) and the others (prim_pairs_fp64[6]: in FP64, or in the
+ * double-single arithmetic of DFJK_MIXED).  Each meets every
  * aux primitive once (one primitive triple).  Either pointer may be NULL.   */
 int dfjk_query_pair_classes(dfjk_handle h, int64_t *prim_pairs_fp64, int64_t *prim_pairs_fp32);
 
 /* The launch-shape choices a handle took from its tuning table, vals[4] =
- * {slicing rows per block, B slicing rows per block, K GEMM split-K
+ * {slicing rows per block, B slicing warps per block, K GEMM split-K
  * range in MB, build work-buffer cap in MB}; 0 = the built-in default.       */
 int dfjk_query_tuning(dfjk_handle h, int32_t *vals);
 
 /* Layout of a handle's setup: the number of 3-centre column slabs (T is
- * built and whitened slab by slab, at most 4 GiB each, 2 GiB in the mixed
- * path) and whether B holds rows for the Schwarz-kept AO pairs only (1 for
- * every DFJK_MIXED handle; 0 for DFJK_FP64, whose B has both triangles of
- * every pair).  Either output pointer may be NULL.                           */
+ * built and whitened slab by slab, at most 4 GiB each, 2 GiB where the
+ * whitening is a sliced product) and whether B holds rows for the Schwarz-kept
+ * AO pairs only (1 for every DFJK_MIXED handle; 0 for DFJK_FP64, whose B has
+ * both triangles of every pair).  Either output pointer may be NULL.        */
 int dfjk_query_setup(dfjk_handle h, int32_t *nslab, int32_t *lean);
 
 /* Aux-row chunking of the DFJK_MIXED build (the build slices B, forms X and
  * adds its K contribution chunk by chunk of rows P, one X and one K GEMM
  * launch per chunk): rows per chunk and the number of chunks, both 0 before
- * the handle's first build and for DFJK_FP64.  Either pointer may be NULL.   */
+ * the handle's first build and for DFJK_FP64, whose builds work in such chunks
+ * too (above nao^2 naux = 3e5) but do not report them.  Either pointer may be
+ * NULL.                                                                      */
 int dfjk_query_build(dfjk_handle h, int32_t *chunk_rows, int32_t *nchunk);
 
 /* Device bytes a molecule with nao AOs and naux aux functions takes at the
@@ -206,7 +213,8 @@ int dfjk_query_build(dfjk_handle h, int32_t *chunk_rows, int32_t *nchunk);
  * inverse; for DFJK_MIXED an upper bound that counts every mu >= nu pair as
  * kept, dfjk_query gives a set-up handle's actual bytes), `build_ws` = the
  * work buffers a build at nocc occupied orbitals
- * adds (kept by the handle for its next builds), `setup_ws` = the transient
+ * adds (kept by the handle for its next builds; without the staging buffer of
+ * b_on_host, one chunk's columns of B), `setup_ws` = the transient
  * peak of the setup beyond the resident data (released when it returns).
  * Used to admit molecules under a memory budget (batching, serving).
  * Any output pointer may be NULL.  Errors: DFJK_ERR_ARG.                     */
@@ -232,10 +240,13 @@ int dfjk_build(dfjk_handle h, int32_t nset, int32_t nocc, const double *C_occ,
  *   D    : device, nset x nao x nao FP64, symmetric.
  *   J, K : device, nset x nao x nao FP64.
  *   E_J, E_K : nset doubles each, Tr(D J)/2 and Tr(D K)/2, host or device.
- * Uses a work buffer of nao^2 naux_pad doubles for the duration of the call,
- * and for a DFJK_MIXED handle (B of the kept pairs only) a second one holding
- * B in both triangles of every pair; synchronises the stream before
- * returning.  Errors: DFJK_ERR_ARG, _OOM, _TIMEOUT, _CUDA.                   */
+ * For the duration of the call it holds W = B D for a range of one AO index
+ * (nao naux_pad doubles per value of it), the slices of W and of B for the range
+ * (twice as much each), together about 8 GiB or 64 values, and the slices of the
+ * kept pairs of B (at most DFJK_BUILD_WS_MB); below nao^2 naux = 3e5, W alone for
+ * the whole range.  For a DFJK_MIXED handle (B of the kept pairs only) also B in
+ * both triangles of every pair.  Synchronises the stream before returning.
+ * Errors: DFJK_ERR_ARG, _OOM, _TIMEOUT, _CUDA.                               */
 int dfjk_build_density(dfjk_handle h, int32_t nset, const double *D, double *J, double *K,
                        double *E_J, double *E_K, void *stream);
 
@@ -246,9 +257,13 @@ int dfjk_build_density(dfjk_handle h, int32_t nset, const double *D, double *J, 
  * (SCF, gradient, Hessian), computed as
  *   dE_J/dR = sum_P d_P du_P/dR - d^T (dV/dR) d / 2,   d = V^-1 u = L^-T rho,
  * with derivative 3-centre and 2-centre integrals over the kept shell pairs:
- * FP64, except that a DFJK_MIXED handle evaluates the pairs whose integrals
- * its build evaluates in FP32 (Schwarz bound below fp32_pair_thresh) in FP32
- * too, accumulated in FP64.  The AO density is
+ * FP64 for DFJK_FP64.  A DFJK_MIXED handle evaluates the pairs whose integrals
+ * its build evaluates in FP32 (Schwarz bound below fp32_pair_thresh) in FP32 and
+ * the others in double-single arithmetic (about 48 bits), as it does their
+ * integrals, sums a block's contributions in double-single and the blocks' in
+ * FP64; fp32_pair_thresh = 0, a basis or geometry outside the double-single range
+ * (dfjk_precision) and densities or fitted coefficients outside 2^-40 .. 2^30 take
+ * FP64.  The atomic sums make repeated calls differ by rounding.  The AO density is
  * held fixed (no orbital response or overlap-derivative term: those belong to
  * the full SCF gradient, not to the Coulomb build).
  *   D    : device nao x nao FP64, symmetric (e.g. C C^T).
@@ -264,12 +279,16 @@ int dfjk_coulomb_gradient(dfjk_handle h, const double *D, double *grad, void *st
  *   dE/dR = sum_P Tr(G_P dT_P/dR) - Tr(W dV/dR) / 2,
  * G_P = d_P D (J) or C Z_P C^T (K), W = d d^T (J) or Z Z^T (K), with
  * Z_P = sum_Q (L^-1)_QP C^T B_Q C (nocc x nocc per aux function).  The
- * derivative integrals are FP64 when c_k != 0 (with c_k = 0 the precision
- * split of dfjk_coulomb_gradient applies); the K part's contractions (X = B C, C^T X,
- * Z, Z Z^T, C Z_P C^T) run with the build's products, the exact slices of the
+ * derivative integrals are FP64 for DFJK_FP64 and double-single for every pair of
+ * a DFJK_MIXED handle, weights included (FP64 where dfjk_coulomb_gradient takes
+ * it; with c_k = 0 the precision split of that call applies); the K part's
+ * contractions (X = B C, C^T X, Z, Z Z^T, C Z_P C^T) run with the build's
+ * products, the exact slices of the
  * handle's precision (or the FP64 pipe for DFJK_FP64's small molecules).
- * The K part holds Z, W (naux_pad^2) and G (naux_pad x nao^2 doubles, the
- * size of B), plus their sliced forms, for the duration of the call.
+ * The K part holds X (naux_pad nao nocc doubles), C^T X and Z (naux_pad nocc^2
+ * each), W (naux_pad^2) and G (naux_pad x nao^2), slices of them within about the
+ * build's work buffers, then the weights of the kept pairs (naux_pad doubles per
+ * kept AO pair).
  *   C_occ : device nao x nocc FP64 row-major, 1 <= nocc <= nao.
  *   c_j, c_k : finite weights of E_J and E_K (c_k = 0 skips the K part).
  *   grad : device natom x 3 FP64, overwritten.

@@ -458,9 +458,11 @@ void enumerate_pairs(dfjk_ctx *h) {
 // cores, some 40 TFLOP/s of FP64-grade work against the FP64 pipe's 1.06, once
 // nao^2 naux reaches this (one build at 4 atoms, 6.9e5: 345 us on the FP64 pipe,
 // 216 us here; at 20 atoms 12.8 and 1.0 ms, whitening 14.2 and 0.96); the water
-// input (2e4) takes 183 us on the FP64 pipe and 186 us here.  The errors of J, K and
-// the gradient against 64-bit references are the FP64 pipe's to three digits at 6
-// to 28 atoms (J 1e-13 to 3e-12 relative): T, V and L^-1 set them.
+// input (2e4) takes 183 us on the FP64 pipe and 186 us here.  Errors against 64-bit
+// references, geometric means of the largest relative ones: 24 molecules of 5 to 23 atoms
+// J 3.7e-12 and K 4.4e-13 (FP64 pipe and an earlier Cholesky: 3.4e-12 and 4.6e-13); 32 of 5
+// to 10 atoms, gradient of E_J - E_K/2, 2.63e-12 here and on the FP64 pipe (2.87e-12
+// before).  V, T and L^-1 set them; one molecule alone goes either way by a factor of two.
 constexpr double OZ_F64_MIN_WORK = 3e5;
 bool use_slices(int precision, int nao, int np) {
   return precision == DFJK_MIXED || (double)nao * nao * np >= OZ_F64_MIN_WORK;

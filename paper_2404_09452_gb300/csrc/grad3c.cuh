@@ -25,8 +25,10 @@
 // whose integrals the build takes in FP32.  Measured: E_J gradient
 // at 45 atoms 33.5 -> 12.4 ms (FP64 and FP32 before; 9.7 with the classes on
 // streams), E_J - E_K/2 at 30 atoms 60 -> 20.6 ms (16.1), FP64 handle at 12 atoms
-// 23.3 -> 6.7 ms; errors of mixed handles against FP64 ones as before (E_J at 9 to
-// 45 atoms 4e-13 to 4e-12, E_J - E_K/2 1e-9 to 4e-9).
+// 23.3 -> 6.7 ms.  Errors of E_J gradients of mixed handles against 64-bit references (32
+// molecules of 6 to 24 atoms, geometric mean of the largest relative ones): 6.8e-12; 6.7e-12
+// with these kernels in FP64, 6.6e-12 with the integrals of the setup in FP64 as
+// well, 7.5e-12 for the kernels before (the metric sets them); E_J - E_K/2 1.0e-9 as before.
 #pragma once
 
 #include "grad.cuh"
