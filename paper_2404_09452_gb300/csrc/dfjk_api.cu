@@ -1187,13 +1187,17 @@ void ensure_workspace(dfjk_ctx *h, int nocc, int nset) {
 
 // After the stream of a call has been synchronised: an expired bounded wait left part of
 // its results unwritten.  The status bit is cleared, so that the next call starts afresh.
-void throw_on_timeout(dfjk_ctx *h, const char *what) {
-  int status = 0;
-  DFJK_CUDA_CHECK(cudaMemcpy(&status, h->status.p, sizeof(int), cudaMemcpyDeviceToHost));
+void throw_on_timeout(dfjk_ctx *h, int status, const char *what) {
   if (status & STATUS_TIMEOUT) {
     DFJK_CUDA_CHECK(cudaMemset(h->status.p, 0, sizeof(int)));
     throw Error{DFJK_ERR_TIMEOUT, std::string("a bounded device wait expired during the ") + what};
   }
+}
+
+void throw_on_timeout(dfjk_ctx *h, const char *what) {
+  int status = 0;
+  DFJK_CUDA_CHECK(cudaMemcpy(&status, h->status.p, sizeof(int), cudaMemcpyDeviceToHost));
+  throw_on_timeout(h, status, what);
 }
 
 __global__ void split_energies_kernel(const double *e, int nset, double *EJ, double *EK) {
@@ -1362,7 +1366,7 @@ void build_one(dfjk_ctx *h, int nocc, const double *C, double *J, double *Kout, 
 struct DensityWork {
   bool sliced = false;
   const double *Bf = nullptr;  // B with both triangles of every pair
-  DBuf<double> Bfull, W, Kpart, stage;
+  DBuf<double> Bfull, W, Kpart, stage, e;
   int ksplit = 1;
   // sliced: X for a range of sigma, the slices of X and B, the lists and exponents
   PairLists pl;
@@ -1780,9 +1784,10 @@ int dfjk_build_density(dfjk_handle h, int32_t nset, const double *D, double *J, 
     rho.alloc(np);
     work.alloc((size_t)RHO_PARTS * np);
     en.alloc(2 * 256);
-    if (!h->e.p || h->e.n < (size_t)(2 * nset)) h->e.alloc(2 * nset);
     DensityWork dw;
     const StreamDrain drain{st};
+    DBuf<double> &e = dw.e;  // energies, then the status word: one read-back for both
+    e.alloc(2 * nset + 1);
     density_work(h, dw, st);
     for (int s = 0; s < nset; ++s) {
       const double *Ds = D + s * nao2;
@@ -1795,7 +1800,7 @@ int dfjk_build_density(dfjk_handle h, int32_t nset, const double *D, double *J, 
       if (dw.sliced) density_k_sliced(h, dw, Ds, Ks, s > 0, st);
       else density_k_f64(h, dw, Ds, Ks, st);
       PhaseScope pe(7, st);
-      energies_f64(Ds, Js, Ks, nao, h->e.p + 2 * s, en.p, st);
+      energies_f64(Ds, Js, Ks, nao, e.p + 2 * s, en.p, st);
     }
     cudaPointerAttributes pa{}, pb{};
     DFJK_CUDA_CHECK(cudaPointerGetAttributes(&pa, EJ));
@@ -1804,19 +1809,23 @@ int dfjk_build_density(dfjk_handle h, int32_t nset, const double *D, double *J, 
     const bool dev_k = pb.type == cudaMemoryTypeDevice || pb.type == cudaMemoryTypeManaged;
     if (dev_j != dev_k) throw Error{DFJK_ERR_ARG, "E_J and E_K must both be host or both device memory"};
     if (dev_j) {
-      split_energies_kernel<<<ceil_div(nset, 64), 64, 0, st>>>(h->e.p, nset, EJ, EK);
+      split_energies_kernel<<<ceil_div(nset, 64), 64, 0, st>>>(e.p, nset, EJ, EK);
       DFJK_LAUNCHED();
-      DFJK_CUDA_CHECK(cudaStreamSynchronize(st));  // W is released on return
-    } else {
-      std::vector<double> e(2 * nset);
-      DFJK_CUDA_CHECK(cudaMemcpyAsync(e.data(), h->e.p, e.size() * sizeof(double), cudaMemcpyDeviceToHost, st));
-      DFJK_CUDA_CHECK(cudaStreamSynchronize(st));
-      for (int s = 0; s < nset; ++s) {
-        EJ[s] = e[2 * s];
-        EK[s] = e[2 * s + 1];
-      }
     }
-    if (dw.sliced) throw_on_timeout(h, "density build");  // the FP64 pipe has no bounded waits
+    std::vector<double> back(2 * nset + 1, 0.0);
+    const size_t n = dw.sliced ? back.size() : back.size() - 1;  // the FP64 pipe has no bounded waits
+    if (dw.sliced) DFJK_CUDA_CHECK(cudaMemcpyAsync(e.p + 2 * nset, h->status.p, sizeof(int), cudaMemcpyDeviceToDevice, st));
+    if (!dev_j || dw.sliced)
+      DFJK_CUDA_CHECK(cudaMemcpyAsync(back.data(), e.p, n * sizeof(double), cudaMemcpyDeviceToHost, st));
+    DFJK_CUDA_CHECK(cudaStreamSynchronize(st));
+    if (!dev_j)
+      for (int s = 0; s < nset; ++s) {
+        EJ[s] = back[2 * s];
+        EK[s] = back[2 * s + 1];
+      }
+    int status;
+    std::memcpy(&status, &back[2 * nset], sizeof(int));
+    throw_on_timeout(h, status, "density build");
     return DFJK_OK;
   } catch (const Error &e) {
     return fail(e);
@@ -1833,7 +1842,7 @@ struct GradWork {
   DBuf<double> rec, gm;  // pair records and weights: doubles or double-single pairs
   DBuf<long long> goff;
   DBuf<int> orb_atom, aux_atom, aux_l;
-  DBuf<unsigned> top;  // high words of the largest |D|, |d|, |C|, |Z|
+  DBuf<unsigned> top;  // high words of the largest |D|, |d|, |C|, |Z|, and the status word
   XWork xw;
   std::deque<SlicedOp> ops;  // slices of the tensor-core GEMMs
   void free_ops() {
@@ -1932,7 +1941,7 @@ static void jk_gradient(dfjk_ctx *h, const double *Din, int nocc, const double *
   AbsMax am{};
   am.x[0] = D; am.n[0] = (long long)nao * nao;
   am.x[1] = d.p; am.n[1] = h->naux;
-  wk.top.alloc(4);
+  wk.top.alloc(5);
   if (exch) {
     // the build's slices on the tensor cores, or FP64 CUDA-core GEMMs for the small
     // molecules of DFJK_FP64
@@ -2103,8 +2112,9 @@ static void jk_gradient(dfjk_ctx *h, const double *Din, int nocc, const double *
     }
   };
   run(h->use_df);
-  unsigned top[4] = {0, 0, 0, 0};
-  if (h->use_df) DFJK_CUDA_CHECK(cudaMemcpyAsync(top, wk.top.p, sizeof(top), cudaMemcpyDeviceToHost, st));
+  unsigned top[5];
+  DFJK_CUDA_CHECK(cudaMemcpyAsync(wk.top.p + 4, h->status.p, sizeof(int), cudaMemcpyDeviceToDevice, st));
+  DFJK_CUDA_CHECK(cudaMemcpyAsync(top, wk.top.p, sizeof(top), cudaMemcpyDeviceToHost, st));
   DFJK_CUDA_CHECK(cudaStreamSynchronize(st));
   if (h->use_df) {
     const double Dm = abs_max_value(top[0]), dm = std::fabs(cj) * abs_max_value(top[1]), Cm = abs_max_value(top[2]);
@@ -2116,7 +2126,7 @@ static void jk_gradient(dfjk_ctx *h, const double *Din, int nocc, const double *
       DFJK_CUDA_CHECK(cudaStreamSynchronize(st));
     }
   }
-  throw_on_timeout(h, "gradient");
+  throw_on_timeout(h, (int)top[4], "gradient");
 }
 
 int dfjk_coulomb_gradient(dfjk_handle h, const double *D, double *grad, void *stream) {
