@@ -74,7 +74,7 @@ def eri_roofline(h, m, ms64, ms32, fp64_peak, fp32_peak, big="fp64"):
     of the pairs above the FP32 threshold; double-single ("df") runs on the FP32
     pipe, beside the FP32 pairs and within the same span ms64."""
     per = eri_flops_per_triple()
-    if not per:
+    if not any(k[3] == big for k in per):
         return None
     naux_prims = [sum(len(sh.exps) for sh in m.aux.shells if sh.l == lc) for lc in range(3)]
     f64 = f32_s = f32_d = df_s = 0.0
@@ -545,7 +545,7 @@ def run_ours(args):
                 "unit": "TFLOP/s", "peak": bf16_sust / prods,
                 "peak_source": f"measured sustained BF16 dense {bf16_sust} TFLOP/s of measured "
                                f"(MEASURED_PEAKS.json) / {prods} exact slice products",
-                "tensor_pipe_tflops": achieved * prods, "traffic": recorded_traffic(dom, args.workload),
+                "tensor_pipe_tflops": achieved * prods, "traffic": None if fp64 else recorded_traffic(dom, args.workload),
                 "algorithmic_flops_per_launch": flops[dom] / nl, "ms_per_launch": dom_ms,
                 "algorithmic_bytes_per_launch": None if fp64 else gemm_bytes[dom] / nl,
                 "launches_per_step": nl}
