@@ -1043,16 +1043,18 @@ size_t build_ws_bytes(int ws_mb) {
   }();
   return ws_mb > 0 ? (size_t)ws_mb << 20 : cap_env;
 }
-// Rows P per chunk of the build: the largest multiple of 128 whose work buffers
-// (X in FP64 and its slices, the slices of B's kept pairs: `steps` K steps of 16
-// over all AOs) stay within DFJK_BUILD_WS_MB megabytes (default 8192), at least
-// 128, at most the whole (padded) aux range.
-int build_chunk_rows(int nao, int np, int nocc, int fmt, long long steps, int ws_mb = 0) {
-  const size_t cap = build_ws_bytes(ws_mb);
+// Bytes that a row P of a chunk takes: X in FP64 and its slices, the slices of B's
+// kept pairs (`steps` K steps of 16 over all AOs).
+size_t chunk_row_bytes(int nao, int nocc, int fmt, long long steps) {
   const size_t rp = ((size_t)nao + OZ_BM - 1) / OZ_BM * OZ_BM;
   const size_t el = 2 * (size_t)oz_slices(fmt);  // bytes of an element's slices
-  const size_t per_row = (size_t)nao * nocc * 8 + rp * nocc * el + (size_t)steps * OZ_BK * el;
-  size_t rows = std::max<size_t>(128, cap / per_row / 128 * 128);
+  return (size_t)nao * nocc * 8 + rp * nocc * el + (size_t)steps * OZ_BK * el;
+}
+// Rows P per chunk of the build: the largest multiple of 128 whose work buffers stay
+// within DFJK_BUILD_WS_MB megabytes (default 8192), at least 128, at most the whole
+// (padded) aux range.
+int build_chunk_rows(int nao, int np, int nocc, int fmt, long long steps, int ws_mb = 0) {
+  size_t rows = std::max<size_t>(128, build_ws_bytes(ws_mb) / chunk_row_bytes(nao, nocc, fmt, steps) / 128 * 128);
   return (int)std::min<size_t>(rows, (size_t)np);
 }
 
@@ -1621,11 +1623,12 @@ int dfjk_estimate_bytes(int32_t nao, int32_t naux, int32_t nocc, int32_t precisi
                    (sl ? n * rup(np, OZ_BM) * ((n + kb - 1) / kb) * 4 + 2 * steps * OZ_BK * 4 : 0);
   size_t ws = n * n * 8 + np * 8 * 2;  // D, rho
   if (sl) {
-    const size_t pc = (size_t)build_chunk_rows(nao, (int)np, nocc, fmt, (long long)steps);
-    const size_t kt = pc * no, nkb = (kt + kb - 1) / kb;
-    ws += n * pc * no * 8 + RHO_PARTS * np * 8;                           // X of a chunk, rho partials
-    ws += oz_slices(fmt) * rup(n, OZ_BM) * rup(kt, OZ_BK) * 2 + rup(n, OZ_BM) * nkb * 4;  // X slices
-    ws += oz_pairs_bytes(fmt, (long long)steps, (int)pc);                 // B slices
+    // X, its slices and the slices of B for a chunk: fewer kept pairs make the chunk
+    // longer, so the cap is the bound unless the whole aux range fits (or 128 rows do not)
+    const size_t row = chunk_row_bytes(nao, nocc, fmt, (long long)steps);
+    const size_t nkb = (np * no + kb - 1) / kb;
+    ws += std::min(row * rup(np, OZ_BM), std::max(build_ws_bytes(0), row * OZ_BM)) + RHO_PARTS * np * 8;
+    ws += rup(n, OZ_BM) * (2 * oz_slices(fmt) * OZ_BK + nkb * 4);         // X slices' padding, exponents
     const size_t cs = c_step_bytes(fmt, nocc);                            // C slices
     ws += std::min(std::max(C_SLICE_CAP, rup(n, OZ_BK) / OZ_BK * cs), steps * cs);
     ws += k_part_doubles(k_shape(nao, fmt, 0), (int)nkb) * 8 + oz_tile_seq_count(nao, nao) * 4;  // K partials
