@@ -229,7 +229,8 @@ int dfjk_estimate_bytes(int32_t nao, int32_t naux, int32_t nocc, int32_t precisi
  *   E_J, E_K : nset doubles each, both host or both device memory (detected;
  *              host memory makes the call synchronise the stream).
  * An expired bounded wait is DFJK_ERR_TIMEOUT; with energies in device memory, which
- * leaves the stream running, the handle's next call that synchronises reports it.
+ * leaves the stream running, the handle's next build or gradient that synchronises
+ * reports it.
  * Work buffers are owned by the handle and reused across calls; calls on one
  * handle must therefore be ordered on a stream.                              */
 int dfjk_build(dfjk_handle h, int32_t nset, int32_t nocc, const double *C_occ,

@@ -1096,6 +1096,7 @@ struct XArgs {
   int mode;
   bool first;
   bool keep_b = false;  // B's slices of these rows are in place already
+  int *status = nullptr;  // status word of the call (null: the handle's)
 };
 void x_gemm_sliced(dfjk_ctx *h, const PairLists &pl, const int *expo, XWork &w, const XArgs &a, cudaStream_t st) {
   const int nao = h->nao;
@@ -1126,7 +1127,7 @@ void x_gemm_sliced(dfjk_ctx *h, const PairLists &pl, const int *expo, XWork &w, 
     x.z0 = h->gfirst_h[g0]; x.nz = h->gfirst_h[g1] - x.z0; x.g0 = g0;
     x.zstep = pl.zstep; x.zgroup = pl.zgroup; x.gstep = pl.gstep;
     x.mode = a.mode; x.out = a.out; x.ldo = a.ldo; x.out_bs = a.obs;
-    x.status = h->status.p; x.timeout = h->opt.timeout_iters;
+    x.status = a.status ? a.status : h->status.p; x.timeout = h->opt.timeout_iters;
     x.tile_ctr = h->tctr.p;
     x.phase = 9;
     oz_gemm(A, c, x, st);
@@ -1236,14 +1237,14 @@ void add_inplace(double *y, const double *x, long long n, cudaStream_t st) {
 // -> 226 us).  The one-tile-per-CTA kernel always writes partials.
 // `w`: from alloc_kwork for at least this range.
 void k_gemm_sliced(dfjk_ctx *h, KWork &w, const SlicedOp &xs, const SlicedOp &ys, int nao, long long kt, double *Kout,
-                   bool add, cudaStream_t st) {
+                   bool add, int *status, cudaStream_t st) {
   const KShape s = k_shape(nao, xs.fmt, h->tune.k_range_mb);
   const KSplit p = k_split(s, xs.nkb);
   if (p.partials ? w.part.n < (size_t)p.n * nao * nao : w.seq.n < oz_tile_seq_count(nao, nao))
     throw Error{DFJK_ERR_STATE, "K work buffers"};
   OzGemmArgs k;
   k.M = nao; k.N = nao; k.K = (int)kt; k.nz = p.n; k.kb_per_split = p.per; k.lower_only = 1;
-  k.status = h->status.p; k.timeout = h->opt.timeout_iters;
+  k.status = status; k.timeout = h->opt.timeout_iters;
   k.tile_ctr = h->tctr.p;
   k.phase = 10;
   if (!p.partials) {
@@ -1355,7 +1356,7 @@ void build_one(dfjk_ctx *h, int nocc, const double *C, double *J, double *Kout, 
       PhaseScope ph(5, st);
       SlicedOp xs = oz_view(h->Xsl, nao, (int)kt);  // rows mu, K (p, i)
       oz_slice_f64(Xc, 0, kt, 1, xs, st, h->tune.slice_rows);
-      k_gemm_sliced(h, h->kw, xs, xs, nao, kt, Kout, c > 0, st);
+      k_gemm_sliced(h, h->kw, xs, xs, nao, kt, Kout, c > 0, h->status.p, st);
     }
     mirror_lower_f64(Kout, nao, st);
     side.join();  // D and J ready
@@ -1378,6 +1379,7 @@ struct DensityWork {
   KWork kw;
   SlicedOp xs, bs;
   int ns = 0, pc = 0;  // sigma and rows P per chunk
+  int *status = nullptr;  // the call's own status word, behind the energies
   ~DensityWork() {
     oz_free(xs);
     oz_free(bs);
@@ -1443,7 +1445,7 @@ void density_k_sliced(dfjk_ctx *h, DensityWork &w, const double *D, double *Kout
         if (h->B.host && !keep_a) b = stage_columns(h, w.stage, p0, pc, st);
         x_gemm_sliced(h, w.pl, w.expo, w.xw,
                       XArgs{b, h->B.host ? pc : h->ldb, D + (long long)s0 * nao, 1, nao, ns, p0, pc, w.W.p + p0, np, kt, 3,
-                            p0 == 0, keep_a || (w.pc >= np && s0 > 0)},
+                            p0 == 0, keep_a || (w.pc >= np && s0 > 0), w.status},
                       st);
       }
     }
@@ -1452,7 +1454,7 @@ void density_k_sliced(dfjk_ctx *h, DensityWork &w, const double *D, double *Kout
     oz_slice_f64(w.W.p, 0, kt, 1, xs, st, h->tune.slice_rows);
     if (!keep_b)
       oz_slice_f64(w.Bf + (long long)s0 * h->ldb, 0, (long long)nao * h->ldb, 1, bs, st, h->tune.slice_rows);
-    k_gemm_sliced(h, w.kw, xs, bs, nao, kt, Kout, s0 > 0, st);
+    k_gemm_sliced(h, w.kw, xs, bs, nao, kt, Kout, s0 > 0, w.status, st);
   }
   mirror_lower_f64(Kout, nao, st);
 }
@@ -1791,6 +1793,8 @@ int dfjk_build_density(dfjk_handle h, int32_t nset, const double *D, double *J, 
     const StreamDrain drain{st};
     DBuf<double> &e = dw.e;  // energies, then the status word: one read-back for both
     e.alloc(2 * nset + 1);
+    dw.status = reinterpret_cast<int *>(e.p + 2 * nset);
+    DFJK_CUDA_CHECK(cudaMemsetAsync(dw.status, 0, sizeof(double), st));
     density_work(h, dw, st);
     for (int s = 0; s < nset; ++s) {
       const double *Ds = D + s * nao2;
@@ -1815,11 +1819,8 @@ int dfjk_build_density(dfjk_handle h, int32_t nset, const double *D, double *J, 
       split_energies_kernel<<<ceil_div(nset, 64), 64, 0, st>>>(e.p, nset, EJ, EK);
       DFJK_LAUNCHED();
     }
-    std::vector<double> back(2 * nset + 1, 0.0);
-    const size_t n = dw.sliced ? back.size() : back.size() - 1;  // the FP64 pipe has no bounded waits
-    if (dw.sliced) DFJK_CUDA_CHECK(cudaMemcpyAsync(e.p + 2 * nset, h->status.p, sizeof(int), cudaMemcpyDeviceToDevice, st));
-    if (!dev_j || dw.sliced)
-      DFJK_CUDA_CHECK(cudaMemcpyAsync(back.data(), e.p, n * sizeof(double), cudaMemcpyDeviceToHost, st));
+    std::vector<double> back(2 * nset + 1);
+    DFJK_CUDA_CHECK(cudaMemcpyAsync(back.data(), e.p, e.bytes(), cudaMemcpyDeviceToHost, st));
     DFJK_CUDA_CHECK(cudaStreamSynchronize(st));
     if (!dev_j)
       for (int s = 0; s < nset; ++s) {
@@ -1828,7 +1829,7 @@ int dfjk_build_density(dfjk_handle h, int32_t nset, const double *D, double *J, 
       }
     int status;
     std::memcpy(&status, &back[2 * nset], sizeof(int));
-    throw_on_timeout(h, status, "density build");
+    if (status & STATUS_TIMEOUT) throw Error{DFJK_ERR_TIMEOUT, "a bounded device wait expired during the density build"};
     return DFJK_OK;
   } catch (const Error &e) {
     return fail(e);
